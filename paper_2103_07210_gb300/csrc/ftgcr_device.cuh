@@ -242,16 +242,6 @@ struct Acc<double> {
     p = t;
     s = s + (q + r);
   }
-  // sum over the warp (xor butterfly, identical order in every warp)
-  __device__ __forceinline__ DD warp_sum() const {
-    DD v{p, s};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      DD w{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-      v = dd_add(v, w);
-    }
-    return v;
-  }
 };
 // Plain FP64 accumulation (one fma per element), for the mixed path's outer
 // residual norm: its decisions need FP64 accuracy, not the oracle's
@@ -297,16 +287,126 @@ struct Acc<float> {
   }
 };
 
-// Per-CTA partial sums: each warp contributes its DD sum of every value; the
-// CTA combines the warps' pairs in a fixed binary tree (depth 3 for 8 warps:
-// GB300's FP64 latency makes a serial chain expensive) and writes nv pairs.
-// FP64 path: double-double adds; FP32 path: each warp pair is first rounded to
-// one double, then plain FP64 adds.
+// Sums of doubles across threads in fixed point (FP64 path).  GB300 issues an
+// FP64 warp instruction every 18 cycles per SM whatever the active lanes, so a
+// double-double tree over a CTA (8 warps x 5 levels x 8 operations a value)
+// took 11 us of a 28 us step round on a 64 x 32 grid.  The integer pipe is some 70 times
+// wider: each double's 53-bit mantissa is placed in a 128-bit two's-complement
+// integer whose unit is fixed by the largest exponent among the terms (bits
+// 64..116 hold the largest term, 10 bits above it take the carries of up to
+// 1024 terms), and the integers are added.  A term is cut below 2^-117 of the
+// largest one, where double-double adds err by 2^-106; integer sums do not
+// depend on their order.  Any infinity or NaN among the terms gives NaN.
+struct Fx {
+  unsigned long long lo;
+  long long hi;
+  int e;  // biased exponent of the unit: value = (hi 2^64 + lo) 2^(e - 1075 - 64); kFxNaN: not finite
+};
+constexpr int kFxNaN = 0x4000;
+__device__ __forceinline__ int fx_exp(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e > 0 ? e : 1;  // subnormals share exponent 1, without the implicit bit
+}
+// v += x in units of exponent E >= fx_exp(x).
+__device__ __forceinline__ void fx_add(Fx& v, double x, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int eb = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  m = eb ? m | 0x10000000000000ull : m;
+  const int sh = E - (eb ? eb : 1);
+  // (m 2^64) >> sh
+  unsigned long long h = sh < 64 ? m >> sh : 0ull;
+  unsigned long long l = sh < 64 ? (m << 1) << (63 - sh) : (sh < 128 ? m >> (sh - 64) : 0ull);
+  if ((long long)b < 0) {  // negate
+    l = 0ull - l;
+    h = ~h + (l == 0ull ? 1ull : 0ull);
+  }
+  v.lo += l;
+  v.hi += (long long)(h + (v.lo < l ? 1ull : 0ull));
+}
+// a += b, both brought to the larger exponent.
+__device__ __forceinline__ void fx_merge(Fx& a, Fx b) {
+  const int E = a.e > b.e ? a.e : b.e;
+  auto down = [&](Fx& x) {
+    const int sh = E - x.e;
+    if (sh == 0) return;
+    if (sh < 64)
+      x.lo = (x.lo >> sh) | (((unsigned long long)x.hi << 1) << (63 - sh));
+    else
+      x.lo = (unsigned long long)(x.hi >> (sh < 127 ? sh - 64 : 63));
+    x.hi = sh < 64 ? x.hi >> sh : x.hi >> 63;
+    x.e = E;
+  };
+  down(a);
+  down(b);
+  a.lo += b.lo;
+  a.hi += b.hi + (a.lo < b.lo ? 1ll : 0ll);
+}
+// Sum over the warp, the same in every lane: five integer reductions of
+// 26-bit pieces (32 of which add up within 32 bits).  Every lane's v.e alike.
+__device__ __forceinline__ Fx fx_warp_sum(const Fx& v) {
+  constexpr unsigned M = (1u << 26) - 1u;
+  const unsigned long long u = (unsigned long long)v.hi;
+  const unsigned p0 = (unsigned)v.lo & M, p1 = (unsigned)(v.lo >> 26) & M, p2 = (unsigned)((v.lo >> 52) | (u << 12)) & M,
+                 p3 = (unsigned)(u >> 14) & M, p4 = (unsigned)(u >> 40);
+  const unsigned long long s0 = __reduce_add_sync(0xffffffffu, p0), s1 = __reduce_add_sync(0xffffffffu, p1),
+                           s2 = __reduce_add_sync(0xffffffffu, p2), s3 = __reduce_add_sync(0xffffffffu, p3),
+                           s4 = __reduce_add_sync(0xffffffffu, p4);
+  Fx r{s0, 0ll, v.e};
+  unsigned long long h = 0ull, t;
+  t = s1 << 26;
+  r.lo += t;
+  h += r.lo < t ? 1ull : 0ull;
+  t = s2 << 52;
+  r.lo += t;
+  h += (r.lo < t ? 1ull : 0ull) + (s2 >> 12);
+  h += s3 << 14;
+  h += s4 << 40;
+  r.hi = (long long)h;
+  return r;
+}
+// The value as a double-double (hi the leading 53 bits or so, lo the rest).
+__device__ __forceinline__ DD fx_dd(const Fx& v) {
+  if (v.e >= kFxNaN) return DD{__longlong_as_double(0x7ff8000000000000ll), 0.0};
+  const double d1 = __ll2double_rz(v.hi);  // |hi| < 2^63: hi - d1 is exact below
+  const long long rem = v.hi - __double2ll_rz(d1);  // under 2^11
+  const double d2 = __ll2double_rn((rem << 50) + (long long)(v.lo >> 14));
+  // units: d1 2^(e-1075), d2 2^(e-1075-50)
+  auto scale = [](double x, int s) {  // x 2^s, |s| < 2200, in two exact halves
+    const int a = s / 2, b = s - a;
+    const double f = __longlong_as_double((long long)(1023 + a) << 52), g = __longlong_as_double((long long)(1023 + b) << 52);
+    return (x * f) * g;
+  };
+  return DD{scale(d1, v.e - 1075), scale(d2, v.e - 1075 - 50)};
+}
+
+// Per-CTA partial sums: each warp contributes its sum of every value, the CTA
+// combines the warps' and writes nv pairs.  FP64 path: fixed point (above),
+// one double-double written.  FP32 path: each warp's pair is first rounded to
+// one double, then plain FP64 adds in a fixed binary tree (depth 3 for 8
+// warps: GB300's FP64 latency makes a serial chain expensive).
 struct CtaRed {
-  DD w[kWarps][kNPart];
+  union {
+    DD w[kWarps][kNPart];
+    Fx f[kWarps][kNPart];
+  };
 };
 __device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, DD x) {
   if ((threadIdx.x & 31) == 0) cr.w[threadIdx.x >> 5][v] = x;
+}
+__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const Acc<float>& a) { cta_red_put(cr, v, a.warp_sum()); }
+__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const AccF64& a) { cta_red_put(cr, v, a.warp_sum()); }
+__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const Acc<double>& a) {
+  int E = fx_exp(a.p);
+  if (a.ex) E = max(E, fx_exp(a.s));
+  E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
+  Fx x{0ull, 0ll, E < 0x7ff ? E : kFxNaN};
+  if (E < 0x7ff) {
+    fx_add(x, a.p, E);
+    if (a.ex) fx_add(x, a.s, E);
+    x = fx_warp_sum(x);
+  }
+  if ((threadIdx.x & 31) == 0) cr.f[threadIdx.x >> 5][v] = x;
 }
 template <typename T>
 __device__ __forceinline__ void cta_red_finish(CtaRed& cr, int nv, double* out, int v0 = 0) {
@@ -314,15 +414,12 @@ __device__ __forceinline__ void cta_red_finish(CtaRed& cr, int nv, double* out, 
   if (threadIdx.x >= v0 && threadIdx.x < nv) {
     const int v = threadIdx.x;
     if constexpr (sizeof(T) == 8) {
-      DD t[kWarps];
+      Fx t = cr.f[0][v];
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) t[w] = cr.w[w][v];
-#pragma unroll
-      for (int h = 1; h < kWarps; h <<= 1)
-#pragma unroll
-        for (int w = 0; w + h < kWarps; w += 2 * h) t[w] = dd_add(t[w], t[w + h]);
-      out[2 * v] = t[0].hi;
-      out[2 * v + 1] = t[0].lo;
+      for (int w = 1; w < kWarps; ++w) fx_merge(t, cr.f[w][v]);
+      const DD d = fx_dd(t);
+      out[2 * v] = d.hi;
+      out[2 * v + 1] = d.lo;
     } else {
       double t[kWarps];
 #pragma unroll

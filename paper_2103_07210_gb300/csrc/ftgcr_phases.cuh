@@ -151,9 +151,9 @@ __device__ __forceinline__ int count_losses(const SolveDev<T>& sd, long long ste
 // ------------------------------------------------------------ reductions
 // Deterministic sum over the nt tiles of the partials buffer of the first nv
 // values.  Warp v sums value v: lanes take tiles lane, lane+32, ... (all loads
-// issued first), add them in tile order, then a fixed xor tree.  FP64 path:
-// double-double arithmetic throughout, rounded once; FP32 path: plain FP64
-// (per-tile values are already accurate sums).  Every CTA that works on the
+// issued first).  FP64 path: fixed point, rounded once (double-double trees
+// here took 6 us of every round); FP32 path: added in tile order, then a fixed
+// xor tree, in plain FP64 (per-tile values are already accurate sums).  Every CTA that works on the
 // solve gets bitwise the same numbers.
 // Warps w0..kWarps-1 take part (warp w0 + i sums values i, i + (kWarps - w0),
 // ...); the order within a value is the same whichever warp sums it.
@@ -163,26 +163,63 @@ __device__ __forceinline__ void reduce_partials(const double* part, int nt, int 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp < w0) return;
   for (int v = warp - w0; v < nv; v += kWarps - w0) {
-    DD acc{0.0, 0.0};
-    double acc1 = 0.0;
-    for (int t0 = lane; t0 < nt; t0 += 32 * B) {
-      DD tv[B];
+    if constexpr (sizeof(T) == 8) {
+      // fixed point (see Fx): the tiles' pairs in batches of 32 B
+      Fx sum{0ull, 0ll, 1};
+      for (int t0 = 0; t0 < nt; t0 += 32 * B) {
+        DD tv[B];
+        int E = 1;
 #pragma unroll
-      for (int q = 0; q < B; ++q) {
-        const int tau = t0 + 32 * q;
-        tv[q] = DD{0.0, 0.0};
-        if (tau < nt) {
-          tv[q].hi = __ldcg(part + (long long)tau * kPartStride + 2 * v);
-          tv[q].lo = __ldcg(part + (long long)tau * kPartStride + 2 * v + 1);
+        for (int q = 0; q < B; ++q) {
+          tv[q] = DD{0.0, 0.0};
+          const int tau = t0 + lane + 32 * q;
+          if (tau < nt) {
+            const V16<double> d = ldv(part + (long long)tau * kPartStride + 2 * v);
+            tv[q] = DD{d.v[0], d.v[1]};
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < B; ++q) E = max(E, max(fx_exp(tv[q].hi), fx_exp(tv[q].lo)));
+        E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
+        Fx x{0ull, 0ll, E < 0x7ff ? E : kFxNaN};
+        if (E < 0x7ff) {
+#pragma unroll
+          for (int q = 0; q < B; ++q)
+            if (t0 + 32 * q < nt) {
+              fx_add(x, tv[q].hi, E);
+              fx_add(x, tv[q].lo, E);
+            }
+          x = fx_warp_sum(x);
+        }
+        if (nt <= 32 * B) {
+          sum = x;
+        } else {
+          // room for the carries of up to 4096 batches (2^20 tiles): 12 bits
+          if (x.e < kFxNaN) {
+            x.lo = (x.lo >> 12) | ((unsigned long long)x.hi << 52);
+            x.hi >>= 12;
+            x.e += 12;
+          }
+          fx_merge(sum, x);
         }
       }
-      if constexpr (sizeof(T) == 8) {
+      if (lane == 0) {
+        const DD d = fx_dd(sum);
+        red[v] = d.hi + d.lo;
+      }
+    } else {
+      double acc1 = 0.0;
+      for (int t0 = lane; t0 < nt; t0 += 32 * B) {
+        DD tv[B];
 #pragma unroll
-        for (int h = 1; h < B; h <<= 1)
-#pragma unroll
-          for (int q = 0; q + h < B; q += 2 * h) tv[q] = dd_add(tv[q], tv[q + h]);
-        acc = dd_add(acc, tv[0]);
-      } else {
+        for (int q = 0; q < B; ++q) {
+          const int tau = t0 + 32 * q;
+          tv[q] = DD{0.0, 0.0};
+          if (tau < nt) {
+            tv[q].hi = __ldcg(part + (long long)tau * kPartStride + 2 * v);
+            tv[q].lo = __ldcg(part + (long long)tau * kPartStride + 2 * v + 1);
+          }
+        }
         double t[B];
 #pragma unroll
         for (int q = 0; q < B; ++q) t[q] = tv[q].hi + tv[q].lo;
@@ -192,13 +229,6 @@ __device__ __forceinline__ void reduce_partials(const double* part, int nt, int 
           for (int q = 0; q + h < B; q += 2 * h) t[q] = t[q] + t[q + h];
         acc1 = acc1 + t[0];
       }
-    }
-    if constexpr (sizeof(T) == 8) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        acc = dd_add(acc, DD{__shfl_xor_sync(0xffffffffu, acc.hi, o), __shfl_xor_sync(0xffffffffu, acc.lo, o)});
-      if (lane == 0) red[v] = acc.hi + acc.lo;
-    } else {
       acc1 = warp_sum(acc1);
       if (lane == 0) red[v] = acc1;
     }
@@ -1305,13 +1335,13 @@ __device__ __forceinline__ void step_stencil(const SolveDev<T>& sd, const Ctx<T>
     }
   }
   sub_mark(ps, 2);
-  if (write_e) cta_red_put(ps.cr, 0, an->warp_sum());
+  if (write_e) cta_red_put(ps.cr, 0, *an);
 #pragma unroll
   for (int l = 0; l < KB; ++l)
-    if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l].warp_sum());
+    if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l]);
   if constexpr (kMixed) {
-    cta_red_put(ps.cr, 2 + c.nu, ah.warp_sum());
-    cta_red_put(ps.cr, 3 + c.nu, aq.warp_sum());
+    cta_red_put(ps.cr, 2 + c.nu, ah);
+    cta_red_put(ps.cr, 3 + c.nu, aq);
     cta_red_finish<T>(ps.cr, 4 + c.nu, part_out, write_e ? 0 : 1);
   } else {
     cta_red_finish<T>(ps.cr, 2 + c.nu, part_out, write_e ? 0 : 1);
@@ -1376,7 +1406,7 @@ __device__ __noinline__ void phase_pa_any(const SolveDev<T>& sd, const Ctx<T>& c
     }
     if (mode == 1) {
       store_rows(c.eW, rt.h0, rt.h1, nlon, sm, stride);
-      cta_red_put(ps.cr, 0, an.warp_sum());
+      cta_red_put(ps.cr, 0, an);
       cta_red_finish<T>(ps.cr, 1, part_out);
       return;
     }
@@ -1476,8 +1506,8 @@ __device__ __noinline__ void phase_pb(const SolveDev<T>& sd, const Ctx<T>& c, in
       }
     finish(g, pa, la, ldcg(c.rCw + g));
   }
-  cta_red_put(ps.cr, 0, a0.warp_sum());
-  cta_red_put(ps.cr, 1, a1.warp_sum());
+  cta_red_put(ps.cr, 0, a0);
+  cta_red_put(ps.cr, 1, a1);
   cta_red_finish<T>(ps.cr, 2, part_out);
 }
 
@@ -1515,8 +1545,8 @@ __device__ __noinline__ void phase_restore(const SolveDev<T>& sd, const Ctx<T>& 
     a0.add(rr, ll);
     a1.add(ll, ll);
   }
-  cta_red_put(ps.cr, 0, a0.warp_sum());
-  cta_red_put(ps.cr, 1, a1.warp_sum());
+  cta_red_put(ps.cr, 0, a0);
+  cta_red_put(ps.cr, 1, a1);
   cta_red_finish<T>(ps.cr, 2, part_out);
 }
 
@@ -1691,11 +1721,14 @@ template <typename T>
 __device__ __forceinline__ void init_partials(PhaseSmem& ps, double* part_out, const Acc<T>* an, const Acc<T>* aR,
                                               const Acc<T>& a0, const Acc<T>& a1, bool full, const AccF64* aR64 = nullptr) {
   if (full) {
-    cta_red_put(ps.cr, 0, an->warp_sum());
-    cta_red_put(ps.cr, 1, aR64 ? aR64->warp_sum() : aR->warp_sum());
+    cta_red_put(ps.cr, 0, *an);
+    if (aR64)
+      cta_red_put(ps.cr, 1, *aR64);
+    else
+      cta_red_put(ps.cr, 1, *aR);
   }
-  cta_red_put(ps.cr, 2, a0.warp_sum());
-  cta_red_put(ps.cr, 3, a1.warp_sum());
+  cta_red_put(ps.cr, 2, a0);
+  cta_red_put(ps.cr, 3, a1);
   cta_red_finish<T>(ps.cr, 4, part_out, full ? 0 : 2);
 }
 
@@ -1797,8 +1830,11 @@ __device__ __noinline__ void phase_init_any(const SolveDev<T>& sd, const Ctx<T>&
     init_stencil<T>(sd, c, st, sm, ps, a0, a1, vec);
   }
   if (mode == 1) {
-    cta_red_put(ps.cr, 0, an.warp_sum());
-    cta_red_put(ps.cr, 1, c.rin_R && sizeof(T) == 4 ? aR64.warp_sum() : aR.warp_sum());
+    cta_red_put(ps.cr, 0, an);
+    if (c.rin_R && sizeof(T) == 4)
+      cta_red_put(ps.cr, 1, aR64);
+    else
+      cta_red_put(ps.cr, 1, aR);
     cta_red_finish<T>(ps.cr, 2, part_out);
     return;
   }
@@ -1889,8 +1925,8 @@ __device__ __noinline__ void phase_out(const SolveDev<T>& sd, const Ctx<T>& c, i
       }
     }
   }
-  cta_red_put(ps.cr, 0, so.warp_sum());
-  cta_red_put(ps.cr, 1, sR.warp_sum());
+  cta_red_put(ps.cr, 0, so);
+  cta_red_put(ps.cr, 1, sR);
   cta_red_finish<T>(ps.cr, 2, part_out);
 }
 
@@ -1950,7 +1986,10 @@ __device__ __noinline__ void phase_fin(const SolveDev<T>& sd, const Ctx<T>& c, i
       }
     }
   }
-  cta_red_put(ps.cr, 0, acc.warp_sum());
+  if constexpr (sizeof(T) == 8)
+    cta_red_put(ps.cr, 0, acc);
+  else
+    cta_red_put(ps.cr, 0, DD{0.0, 0.0});  // mixed path: no residual formed here
   cta_red_finish<T>(ps.cr, 1, part_out);
 }
 

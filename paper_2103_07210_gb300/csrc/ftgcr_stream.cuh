@@ -738,19 +738,19 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
     return;
   }
   if (pass == 0) {
-    cta_red_put(ps.cr, 0, an.warp_sum());
+    cta_red_put(ps.cr, 0, an);
 #pragma unroll
     for (int l = 0; l < KB; ++l)
-      if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l].warp_sum());
-    cta_red_put(ps.cr, 2 + c.nu, ah.warp_sum());
-    cta_red_put(ps.cr, 3 + c.nu, aq.warp_sum());
+      if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l]);
+    cta_red_put(ps.cr, 2 + c.nu, ah);
+    cta_red_put(ps.cr, 3 + c.nu, aq);
     cta_red_finish<float>(ps.cr, 4 + c.nu, part_out);
   } else {
 #pragma unroll
     for (int l = 0; l < KB; ++l)
-      if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l].warp_sum());
-    cta_red_put(ps.cr, 2 + c.nu, ah.warp_sum());
-    cta_red_put(ps.cr, 3 + c.nu, aq.warp_sum());
+      if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l]);
+    cta_red_put(ps.cr, 2 + c.nu, ah);
+    cta_red_put(ps.cr, 3 + c.nu, aq);
     cta_red_finish_add(ps.cr, 4 + c.nu, part_out, 1);
   }
   if (threadIdx.x == 0) g_ss.cph = cph;

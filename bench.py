@@ -63,8 +63,8 @@ def sources_hash() -> str:
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2103_07210_gb300", "csrc")
     for f in sorted(os.listdir(d)):
-        if f in ("ftgcr_device.cuh", "ftgcr_phases.cuh", "ftgcr_stream.cuh", "ftgcr_instances.h") or \
-                (f.startswith("ftgcr_k") and f.endswith(".cu")):
+        if f in ("ftgcr_device.cuh", "ftgcr_phases.cuh", "ftgcr_stream.cuh", "ftgcr_band.cuh", "ftgcr_instances.h") or \
+                (f.startswith(("ftgcr_k", "ftgcr_b")) and f.endswith(".cu")):
             h.update(open(os.path.join(d, f), "rb").read())
     return h.hexdigest()
 

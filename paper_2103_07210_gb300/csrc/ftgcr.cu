@@ -16,6 +16,7 @@
 #include "../../include/ftgcr.h"
 #include "ftgcr_device.cuh"
 #include "ftgcr_phases.cuh"
+#include "ftgcr_band.cuh"
 #include "ftgcr_instances.h"
 #include "ftgcr_serve.h"
 
@@ -375,6 +376,27 @@ __global__ void k_lf_pieces(int nlon, int nlat, int C, const double* __restrict_
   }
 }
 
+// Constants in the layout of the banded rounds: row j, plane q, piece p holds
+// the W elements p CQ + q W .. of c = -u, winv, z (zero past the leading block
+// and in the padding), CQ = W 2^lq.
+template <typename O>
+__global__ void k_lf_band(int nlon, int nlat, int lq, int PC, const double* __restrict__ u,
+                          const double* __restrict__ winv, const double* __restrict__ z, O* lc, O* lw, O* lz) {
+  constexpr int W = 16 / sizeof(O);
+  const int Q = 1 << lq, per = Q * PC * W, m = nlon - 1;
+  const long long total = (long long)per * nlat;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total; q += (long long)gridDim.x * blockDim.x) {
+    const int j = (int)(q / per), pos = (int)(q - (long long)j * per);
+    const int un = pos / W, plane = un / PC, p = un - plane * PC;
+    const int i = (p << lq) * W + plane * W + (pos - un * W);
+    const bool in = i < m;
+    const long long g = (long long)j * nlon + i;
+    lc[q] = in ? (O)(-u[g]) : O(0);
+    lw[q] = in ? (O)winv[g] : O(0);
+    lz[q] = in ? (O)z[g] : O(0);
+  }
+}
+
 // The line preconditioner's factorisation (Jacobi: its diagonal), enqueued
 // on st.  FP64 outputs l, winv, u, z (z doubles as scratch for the diagonal)
 // and the row constants; FP32 chunk-layout constants when lc32 is given.
@@ -489,6 +511,8 @@ __global__ void k_begin_solve(SolveDev<T>* sd, BeginArgs b, int* active, int n_a
       S.status = ST_NOT_CONVERGED;
       S.refused = 1;
       *sd->result = S;
+      sd->st[0] = S;
+      sd->st[1] = S;
       active[slot] = 0;
       active[n_active + slot] = 0;
       if (ctl) {
@@ -506,6 +530,7 @@ __global__ void k_begin_solve(SolveDev<T>* sd, BeginArgs b, int* active, int n_a
     sd->xout = b.xout;
     sd->nfaults = b.nfaults;
     sd->nlosses = b.nlosses;
+    sd->solve_id += 1u;
     SolveState S;
     memset(&S, 0, sizeof S);
     S.active = 1;
@@ -659,6 +684,81 @@ SmemPlan smem_plan(int nlon, int nlat, int nt, int mixed, size_t elem, int preco
   return p;
 }
 
+// Banded rounds (ftgcr_band.cuh): the layout of a row and of the shared memory
+// for bands of at most H rows.  Shared memory takes the band's rows with their
+// halo rows and the threads' sums, then, as far as they fit, the rows' line-
+// solve constants, the band's vectors (r, L(e) and up to k L(p^l)) and the
+// rows' face coefficients.
+constexpr int kBandMaxLon = 4095;
+struct BandLayout {
+  int local, lq, NP, NPc, lG, PC, nbuf, cs_staged, ts_staged;
+  int rowb, conb, bufb, faceb, red_off, con_off, ts_off, buf_off, sub_h, mega;
+  size_t bytes;
+};
+constexpr int kOnePassGroups = 1450;  // (see fill_handle_params)
+bool band_layout(int nlon, int nlat, int nt, bool mixed, int k, size_t limit, BandLayout* b) {
+  if (nlon > kBandMaxLon) return false;
+  const int W = mixed ? 4 : 2, elem = 16 / W, H = (nlat + nt - 1) / nt, NG = (nlon + 3) / 4;
+  const long long p8 = (nlon + 7) / 8;
+  auto row = [&](int cq) {  // the layout of a row with pieces of cq elements
+    const int Q = cq / W;
+    b->lq = Q == 2 ? 1 : Q == 4 ? 2 : 3;
+    b->NPc = (nlon + cq - 1) / cq;
+    b->PC = b->NPc;
+    b->lG = 0;
+    while ((32 << b->lG) < b->NPc) ++b->lG;
+    // plane pitch: see BandRow
+    b->NP = b->NPc;
+    while (Q == 8 ? !(b->NP & 1) : (b->NP & 7) != (Q == 2 ? 4 : 2)) ++b->NP;
+    b->rowb = Q * b->NP * 16;
+    b->conb = Q * b->PC * 16;
+    return (32 << b->lG) <= kBandThreads;
+  };
+  // pieces of 8 elements; of 16 where 8 would take a second trip over the
+  // threads (FP32), or more threads than there are (FP64, whose pieces of 16
+  // take more of its registers)
+  const size_t st = (size_t)row_stride(nlon) * sizeof(double), sums = 8 * (size_t)kBandThreads * (k + 3);
+  b->sub_h = 0;
+  size_t out = 0;
+  if (mixed) {  // the refinement round's FP64 rows, in sub-bands
+    if (3 * st > limit) return false;
+    b->sub_h = (int)std::min<size_t>((size_t)H, limit / st - 2);
+    out = (size_t)(b->sub_h + 2) * st;
+  }
+  // local: every vector and the constants, halo rows included, in shared
+  // memory.  The face coefficients where they fit too
+  b->local = 0;
+  if (mixed && row((H + 2) * p8 > kBandThreads ? 16 : 8)) {
+    const size_t vec = (size_t)(H + 2) * NG * 16,
+                 fixed = (size_t)(std::max(1, kBandThreads / (H * NG)) * H + 2) * b->rowb + sums;
+    // (without the constants beside them, measured 2 % slower than the exchange
+    // at 1024 x 512 and 8 % at 1208 x 531)
+    if (fixed + (size_t)(k + 2) * vec + 3 * (size_t)(H + 2) * b->conb <= limit) {
+      b->local = 1;
+      b->bufb = (int)vec;
+    }
+  }
+  if (!b->local) {
+    if (!row((mixed ? H * p8 : p8) > kBandThreads ? 16 : 8)) return false;
+    b->bufb = H * NG * 4 * elem;
+  }
+  b->faceb = H * NG * 4 * elem;
+  b->mega = std::max(1, kBandThreads / (H * NG));
+  b->red_off = (b->mega * H + 2) * b->rowb;
+  const size_t rows = (size_t)b->red_off + sums;
+  if (rows > limit) return false;
+  const size_t con = 3 * (size_t)(H + 2 * b->local) * b->conb, face = (size_t)b->faceb * 2 + (size_t)NG * 4 * elem;
+  const size_t want = (size_t)(b->local ? k + 2 : 2) * b->bufb;
+  b->cs_staged = rows + con + want <= limit;
+  b->con_off = (int)rows;
+  b->ts_off = (int)(rows + (b->cs_staged ? con : 0));
+  b->nbuf = (int)std::min<size_t>((size_t)k + 2, (limit - b->ts_off) / b->bufb);
+  b->ts_staged = b->nbuf == k + 2 && b->ts_off + face + (size_t)b->nbuf * b->bufb <= limit;
+  b->buf_off = b->ts_off + (b->ts_staged ? (int)face : 0);
+  b->bytes = kBandFixed + std::max(out, (size_t)b->buf_off + (size_t)b->nbuf * b->bufb);
+  return true;
+}
+
 // Row bands and round structure of a solve.  Equal-height row bands: the
 // round takes as long as the tallest band, so use the fewest bands of that
 // height (e.g. 512 rows on 152 SMs: 128 x 4), as tall as shared memory allows.
@@ -775,7 +875,9 @@ struct ftgcr_handle {
   SolveDev<float> sd32{};
   size_t smem = 0;
   int split = 0;  // split rounds (see choose_tiling)
-  int wide = 0;   // runs in the wide-row kernel instance (split rounds, or FP64 factors from global memory)
+  int wide = 0;   // kernel instance: 1, 2 wide rows (split or streamed rounds, or FP64 factors from global memory),
+                  // kWideBand banded rounds
+  BandLayout bl{};  // banded rounds
   int noalloc = 0;  // the record of a no-allocation solve (its pool is the static scratch array)
   SmemPlan plan{};
   int grid = 0;
@@ -833,7 +935,7 @@ int occupancy(int kb, int split, size_t smem, int* occ) {
     *occ = it->second;
     return FTGCR_OK;
   }
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, f, kThreads, smem));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, f, split == kWideBand ? kBandThreads : kThreads, smem));
   known[{f, smem}] = *occ;
   return FTGCR_OK;
 }
@@ -881,7 +983,8 @@ size_t layout(ftgcr_handle* h, unsigned char* base, SolveDev<T>* sd) {
   const size_t vT = sizeof(T) * N, v64 = sizeof(double) * N;
   const bool fp64 = std::is_same<T, double>::value;
   // preconditioner arrays: FP64 natural [N] (+ u), FP32 chunk layout [nlat][32 C]
-  const size_t lcn = (h->precond == FTGCR_PRECOND_LINE) ? (fp64 ? (size_t)N : (size_t)nlat * 32 * C)
+  const bool band = h->wide == kWideBand;
+  const size_t lcn = (h->precond == FTGCR_PRECOND_LINE) ? (fp64 ? (size_t)N : band ? 1 : (size_t)nlat * 32 * C)
                                                         : (h->precond == FTGCR_PRECOND_JACOBI ? (size_t)N : 1);
   h->Tx64 = (double*)take(v64);
   h->Ty64 = (double*)take(v64);
@@ -898,22 +1001,25 @@ size_t layout(ftgcr_handle* h, unsigned char* base, SolveDev<T>* sd) {
   // (not with FTGCR_FLAG_ORACLE_ORDER: the oracle's serial order on every row;
   // the shared-memory plan was sized for the larger chunk layout)
   const bool chunk = fp64 && h->precond == FTGCR_PRECOND_LINE && h->nlon >= kChunkMinLon && !h->noalloc &&
-                     !(h->flags & FTGCR_FLAG_ORACLE_ORDER);
+                     !(h->flags & FTGCR_FLAG_ORACLE_ORDER) && !band;
   sd->lchunk = chunk ? 1 : 0;
   sd->lcc = chunk ? (const T*)take(sizeof(T) * 32 * (size_t)C * nlat) : sd->lc;
   sd->lwc = chunk ? (const T*)take(sizeof(T) * 32 * (size_t)C * nlat) : sd->lw;
   sd->lzc = chunk ? (const T*)take(sizeof(T) * 32 * (size_t)C * nlat) : sd->lz;
   // streamed solves: the FP32 constants again in the piece-major layout
+  // (banded solves: in their own layout, in the solve's precision)
   const bool piece = !fp64 && h->split == 2;
-  sd->lcp = piece ? (const T*)take(sizeof(T) * 32 * (size_t)(C + 4) * nlat) : nullptr;
-  sd->lwp = piece ? (const T*)take(sizeof(T) * 32 * (size_t)(C + 4) * nlat) : nullptr;
-  sd->lzp = piece ? (const T*)take(sizeof(T) * 32 * (size_t)(C + 4) * nlat) : nullptr;
+  const size_t pb = band ? (size_t)h->bl.conb * nlat : piece ? sizeof(T) * 32 * (size_t)(C + 4) * nlat : 0;
+  sd->lcp = pb ? (const T*)take(pb) : nullptr;
+  sd->lwp = pb ? (const T*)take(pb) : nullptr;
+  sd->lzp = pb ? (const T*)take(pb) : nullptr;
+  sd->hrow = band ? (uint4*)take((size_t)h->nt * 4 * ((h->nlon + 3) / 4) * 8 * sizeof(T)) : nullptr;
   size_t before = off;
   for (int q = 0; q < 3; ++q) sd->phi[q] = (T*)take(vT);
   for (int q = 0; q < 3; ++q) sd->r[q] = (T*)take(vT);
   sd->e[0] = (T*)take(vT);
   sd->Le[0] = (T*)take(vT);
-  if (std::is_same<T, float>::value) {  // mixed path: fused steps double-buffer e, L(e)
+  if (std::is_same<T, float>::value || band) {  // fused steps double-buffer e, L(e)
     sd->e[1] = (T*)take(vT);
     sd->Le[1] = (T*)take(vT);
   } else {
@@ -989,14 +1095,20 @@ int setup_coefficients(ftgcr_handle* h, const SolveDev<T>& sd, const double* Dd,
     z64 = tmp + 3 * h->N;
     r64 = tmp + 4 * h->N;
   }
-  const bool chunk = !mixed && sd.lchunk;
+  const bool chunk = !mixed && sd.lchunk, c32 = mixed && !sd.band;
   const int frc = launch_line_factor(h->nlon, h->nlat, h->C, h->precond, h->Tx64, h->Ty64, h->muA64, l64, w64, u64,
-                                     z64, r64, mixed ? (float*)sd.lc : nullptr, mixed ? (float*)sd.lw : nullptr,
-                                     mixed ? (float*)sd.lz : nullptr, mixed ? (float*)sd.lrow : nullptr, st,
+                                     z64, r64, c32 ? (float*)sd.lc : nullptr, c32 ? (float*)sd.lw : nullptr,
+                                     c32 ? (float*)sd.lz : nullptr, mixed ? (float*)sd.lrow : nullptr, st,
                                      chunk ? (double*)sd.lcc : nullptr, chunk ? (double*)sd.lwc : nullptr,
-                                     chunk ? (double*)sd.lzc : nullptr, mixed ? (float*)sd.lcp : nullptr,
-                                     mixed ? (float*)sd.lwp : nullptr, mixed ? (float*)sd.lzp : nullptr);
+                                     chunk ? (double*)sd.lzc : nullptr, c32 ? (float*)sd.lcp : nullptr,
+                                     c32 ? (float*)sd.lwp : nullptr, c32 ? (float*)sd.lzp : nullptr);
   if (frc) return frc;
+  if (sd.band) {
+    const long long nb = (long long)(sd.conb / (int)sizeof(T)) * h->nlat;
+    k_lf_band<T><<<(int)std::min<long long>((nb + 255) / 256, 8192), 256, 0, st>>>(
+        h->nlon, h->nlat, sd.lq, sd.PC, u64, w64, z64, (T*)sd.lcp, (T*)sd.lwp, (T*)sd.lzp);
+    CK(cudaGetLastError());
+  }
   CK(cudaFreeAsync(scratch, st));
   return FTGCR_OK;
 }
@@ -1035,6 +1147,17 @@ int create_impl(ftgcr_handle* h, const double* D_host_or_dev, bool D_on_device) 
   sd.cs_global = h->plan.gconsts;
   sd.sub_h = h->plan.sub_h;
   sd.nslot = h->plan.nslot;
+  if (h->wide == kWideBand) {
+    const BandLayout& b = h->bl;
+    sd.band = 1;
+    sd.lq = b.lq, sd.NP = b.NP, sd.NPc = b.NPc, sd.lG = b.lG, sd.PC = b.PC, sd.nbuf = b.nbuf, sd.cs_staged = b.cs_staged;
+    sd.ts_staged = b.ts_staged, sd.ts_off = b.ts_off, sd.local = b.local, sd.faceb = b.faceb;
+    sd.NG = (h->nlon + 3) / 4, sd.rng = 1.0f / (float)sd.NG;
+    sd.rb = h->nlat / h->nt, sd.rx = h->nlat % h->nt, sd.mega = b.mega;
+    sd.rowb = b.rowb, sd.conb = b.conb, sd.bufb = b.bufb, sd.red_off = b.red_off;
+    sd.con_off = b.con_off, sd.buf_off = b.buf_off;
+    sd.sub_h = b.sub_h;
+  }
   sd.Tx64 = h->Tx64;
   sd.Ty64 = h->Ty64;
   sd.muA64 = h->muA64;
@@ -1063,7 +1186,7 @@ int create_impl(ftgcr_handle* h, const double* D_host_or_dev, bool D_on_device) 
     h->sd64 = sd;
 
   (void)mixed;
-  h->smem = h->plan.bytes;
+  h->smem = h->wide == kWideBand ? h->bl.bytes : h->plan.bytes;
   int rc = configure_kernel<T>(kbound(h->k), h->wide, std::max<size_t>(h->smem, 1));
   if (rc) return rc;
   int occ = 0;
@@ -1150,6 +1273,85 @@ int launch_persistent(int kb, SolveDev<T>* const* solves, const int* nt, int* ac
   return FTGCR_OK;
 }
 
+// The banded kernel: one solve over the whole grid (cta, order null), or teams
+// of CTAs with a list of solves each.
+template <typename T>
+int launch_band(int kb, SolveDev<T>* const* solves, int* active, const TeamCta* cta, const int* order,
+                unsigned int* counter, LaunchCtl* ctl, int* diag, int max_rounds, int grid, size_t smem,
+                cudaStream_t st) {
+  BandArgs<T> a;
+  a.solves = solves;
+  a.active = active;
+  a.cta = cta;
+  a.order = order;
+  a.counter = counter;
+  a.ctl = ctl;
+  a.max_rounds = max_rounds;
+  a.trace = trace_ptr(grid, &a.trace_rounds);
+  a.diag = diag;
+  void* args[] = {&a};
+  CK(cudaLaunchCooperativeKernel(kernel_ptr<T>(kb, kWideBand), dim3(grid), dim3(kBandThreads), args, smem, st));
+  return FTGCR_OK;
+}
+
+// Teams of CTAs for a launch of several banded solves.  A team runs its solves
+// one after another, so a solve's rounds wait for nobody else's.  As many
+// teams as keep at least kTeamMin CTAs each (a 1024 x 512 solve on one SM
+// takes eight times a round's fixed cost), at most one per solve; CTAs go to
+// teams by the largest solve each would take, then every solve, largest first,
+// to the team that would finish it soonest.
+constexpr int kTeamMin = 8;
+struct TeamPlan {
+  std::vector<TeamCta> cta;  // [grid]
+  std::vector<int> order;    // solves (indices into the argument), team by team
+  int teams = 0;
+};
+void plan_teams(const std::vector<long long>& points, const std::vector<int>& nt, int sms, TeamPlan* out) {
+  const int n = (int)points.size();
+  std::vector<int> by(n);
+  for (int i = 0; i < n; ++i) by[i] = i;
+  std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return points[a] > points[b]; });
+  const int teams = std::max(1, std::min(n, sms / kTeamMin));
+  // sizes: one CTA each, then one by one to the team with the most points per CTA
+  std::vector<int> size(teams, 1);
+  for (int left = sms - teams; left > 0; --left) {
+    int best = -1;
+    double load = 0;
+    for (int t = 0; t < teams; ++t) {
+      if (size[t] >= nt[by[t]]) continue;
+      const double l = (double)points[by[t]] / size[t];
+      if (best < 0 || l > load) best = t, load = l;
+    }
+    if (best < 0) break;
+    ++size[best];
+  }
+  std::vector<double> busy(teams, 0.0);
+  std::vector<std::vector<int>> list(teams);
+  for (int i : by) {
+    int best = 0;
+    double end = 0;
+    for (int t = 0; t < teams; ++t) {
+      // a round: its points over the team's CTAs, plus a fixed cost worth about 8192 points
+      const double e = busy[t] + (double)points[i] / std::min(size[t], nt[i]) + 8192.0;
+      if (t == 0 || e < end) best = t, end = e;
+    }
+    busy[best] = end;
+    list[best].push_back(i);
+  }
+  out->cta.clear();
+  out->order.clear();
+  out->teams = 0;
+  for (int t = 0; t < teams; ++t) {
+    if (list[t].empty()) continue;
+    int most = 1;
+    for (int i : list[t]) most = std::max(most, nt[i]);
+    const int sz = std::min(size[t], most), q0 = (int)out->order.size();
+    for (int i : list[t]) out->order.push_back(i);
+    for (int r = 0; r < sz; ++r) out->cta.push_back(TeamCta{out->teams, r, sz, q0, (int)out->order.size()});
+    ++out->teams;
+  }
+}
+
 BeginArgs begin_args(const ftgcr_handle* h, const double* R, const double* x0, double* xout,
                      const ftgcr_fault_plan* plan) {
   BeginArgs b;
@@ -1174,8 +1376,11 @@ int solve_async_impl(ftgcr_handle* h, const double* R, const double* x0, double*
   CK(cudaGetLastError());
   // every inner step takes two rounds, every refinement sweep a few more
   const int max_rounds = (int)std::min<long long>(1 << 30, 2 * h->max_steps + 8 * ((long long)h->max_outer + 2) + 16);
-  int rc = launch_persistent<T>(kbound(h->k), (SolveDev<T>* const*)h->sdev_arr, h->nt_dev, h->active, 1, h->ctl,
-                                h->diag, max_rounds, h->grid, h->smem, h->wide, st);
+  int rc = h->wide == kWideBand
+               ? launch_band<T>(kbound(h->k), (SolveDev<T>* const*)h->sdev_arr, h->active, nullptr, nullptr,
+                                &h->ctl->counter, h->ctl, h->diag, max_rounds, h->grid, h->smem, st)
+               : launch_persistent<T>(kbound(h->k), (SolveDev<T>* const*)h->sdev_arr, h->nt_dev, h->active, 1, h->ctl,
+                                      h->diag, max_rounds, h->grid, h->smem, h->wide, st);
   if (rc) return rc;
   CK(cudaMemcpyAsync(h->h_result, h->result, sizeof(SolveState), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(h->h_ctl, h->ctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
@@ -1184,77 +1389,122 @@ int solve_async_impl(ftgcr_handle* h, const double* R, const double* x0, double*
   return FTGCR_OK;
 }
 
+// The schedule of a banded launch, filled like the solve table.
+constexpr int kMaxTeamCtas = 256;
+struct TeamTable {
+  TeamCta cta[kMaxTeamCtas];
+  int n;
+};
+__global__ void k_fill_teams(TeamTable t, TeamCta* d_cta) {
+  if ((int)threadIdx.x < t.n) d_cta[threadIdx.x] = t.cta[threadIdx.x];
+}
+
 // Several independent solves in one persistent launch.  Each solve keeps its
 // own handle's tiling and reduction order, so its arithmetic is bitwise that
 // of a lone solve; the launch only interleaves the solves' tiles over the
 // CTAs.  The launch's own arrays (solve pointers, tile counts, active flags,
 // control block, progress record) are stream-ordered allocations freed after
 // the launch, and the solve table is written by a kernel from its parameters
-// (no copy from host memory), so a batch captures into a CUDA graph.
+// (no copy from host memory), so a batch captures into a CUDA graph.  A batch
+// that mixes banded solves with others takes one launch for each kind, one
+// after the other on the stream.
 template <typename T>
-int solve_batch_impl(ftgcr_handle* const* hs, const double* const* rhs, double* const* x,
-                     const ftgcr_fault_plan* const* plans, int n, cudaStream_t st) {
-  int kb = 4;
-  size_t smem = 1;
-  long long max_steps = 0, total_tiles = 0;
-  int max_outer = 0, split = 0;
-  for (int i = 0; i < n; ++i) {
-    split = std::max(split, hs[i]->wide);
-    kb = std::max(kb, kbound(hs[i]->k));
-    smem = std::max(smem, hs[i]->smem);
-    max_steps = std::max(max_steps, hs[i]->max_steps);
-    max_outer = std::max(max_outer, hs[i]->max_outer);
-    total_tiles += hs[i]->nt;
-  }
-  int rc = configure_kernel<T>(kb, split, smem);
-  if (rc) return rc;
-  int occ = 0;
-  rc = occupancy<T>(kb, split, smem, &occ);
-  if (rc) return rc;
-  if (occ < 1) return FTGCR_ERR_ARG;
-  const DeviceInfo di = device_info(hs[0]->dev);
-  const int grid = (int)std::min<long long>(total_tiles, (long long)di.sms * occ);
-  const size_t b_solves = align256(sizeof(void*) * n), b_nt = align256(sizeof(int) * n),
-               b_act = align256(sizeof(int) * 2 * n), b_ctl = align256(sizeof(LaunchCtl)),
-               b_diag = align256(sizeof(int) * 4 * grid);
-  unsigned char* buf = nullptr;
-  CK(cudaMallocAsync((void**)&buf, b_solves + b_nt + b_act + b_ctl + b_diag, st));
-  void** d_solves = (void**)buf;
-  int* d_nt = (int*)(buf + b_solves);
-  int* d_act = (int*)(buf + b_solves + b_nt);
-  LaunchCtl* d_ctl = (LaunchCtl*)(buf + b_solves + b_nt + b_act);
-  int* d_diag = (int*)(buf + b_solves + b_nt + b_act + b_ctl);
-  for (int off = 0; off < n; off += kTableChunk) {
-    BatchTable tb;
-    tb.n = std::min(kTableChunk, n - off);
-    tb.off = off;
-    for (int i = 0; i < tb.n; ++i) {
-      tb.sdev[i] = hs[off + i]->sdev;
-      tb.nt[i] = hs[off + i]->nt;
+int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, double* const* x,
+                     const ftgcr_fault_plan* const* plans, int n_all, cudaStream_t st) {
+  for (int band = 0; band < 2; ++band) {
+    std::vector<int> id;  // this launch's solves
+    int kb = 4;
+    size_t smem = 1;
+    long long max_steps = 0, total_tiles = 0;
+    int max_outer = 0, split = 0;
+    for (int i = 0; i < n_all; ++i) {
+      const ftgcr_handle* h = hs_all[i];
+      if ((h->wide == kWideBand) != (band == 1)) continue;
+      id.push_back(i);
+      split = std::max(split, h->wide);
+      kb = std::max(kb, kbound(h->k));
+      smem = std::max(smem, h->smem);
+      max_steps = std::max(max_steps, h->max_steps);
+      max_outer = std::max(max_outer, h->max_outer);
+      total_tiles += h->nt;
     }
-    k_fill_table<<<1, kTableChunk, 0, st>>>(tb, d_solves, d_nt);
-    CK(cudaGetLastError());
+    const int n = (int)id.size();
+    if (n == 0) continue;
+    int rc = configure_kernel<T>(kb, split, smem);
+    if (rc) return rc;
+    int occ = 0;
+    rc = occupancy<T>(kb, split, smem, &occ);
+    if (rc) return rc;
+    if (occ < 1) return FTGCR_ERR_ARG;
+    const DeviceInfo di = device_info(hs_all[0]->dev);
+    int grid = (int)std::min<long long>(total_tiles, (long long)di.sms * occ);
+    TeamPlan tp;
+    if (band) {
+      std::vector<long long> points;
+      std::vector<int> nts;
+      for (int i : id) {
+        points.push_back(hs_all[i]->N);
+        nts.push_back(hs_all[i]->nt);
+      }
+      plan_teams(points, nts, std::min(di.sms, kMaxTeamCtas), &tp);
+      grid = (int)tp.cta.size();
+    }
+    const size_t b_solves = align256(sizeof(void*) * n), b_nt = align256(sizeof(int) * n),
+                 b_act = align256(sizeof(int) * 2 * n), b_ctl = align256(sizeof(LaunchCtl)),
+                 b_diag = align256(sizeof(int) * 4 * grid), b_cta = align256(sizeof(TeamCta) * tp.cta.size()),
+                 b_cnt = align256(128 * (size_t)tp.teams);
+    unsigned char* buf = nullptr;
+    CK(cudaMallocAsync((void**)&buf, b_solves + b_nt + b_act + b_cnt + b_ctl + b_diag + b_cta, st));
+    void** d_solves = (void**)buf;
+    int* d_nt = (int*)(buf + b_solves);  // banded launch: the teams' order
+    int* d_act = (int*)(buf + b_solves + b_nt);
+    unsigned int* d_cnt = (unsigned int*)(buf + b_solves + b_nt + b_act);
+    LaunchCtl* d_ctl = (LaunchCtl*)(buf + b_solves + b_nt + b_act + b_cnt);
+    int* d_diag = (int*)(buf + b_solves + b_nt + b_act + b_cnt + b_ctl);
+    TeamCta* d_cta = (TeamCta*)(buf + b_solves + b_nt + b_act + b_cnt + b_ctl + b_diag);
+    for (int off = 0; off < n; off += kTableChunk) {
+      BatchTable tb;
+      tb.n = std::min(kTableChunk, n - off);
+      tb.off = off;
+      for (int i = 0; i < tb.n; ++i) {
+        tb.sdev[i] = hs_all[id[off + i]]->sdev;
+        tb.nt[i] = band ? tp.order[off + i] : hs_all[id[off + i]]->nt;
+      }
+      k_fill_table<<<1, kTableChunk, 0, st>>>(tb, d_solves, d_nt);
+      CK(cudaGetLastError());
+    }
+    if (band) {
+      TeamTable tt;
+      tt.n = grid;
+      for (int i = 0; i < grid; ++i) tt.cta[i] = tp.cta[i];
+      k_fill_teams<<<1, kMaxTeamCtas, 0, st>>>(tt, d_cta);
+      CK(cudaGetLastError());
+    }
+    CK(cudaMemsetAsync(d_act, 0, b_act + b_cnt, st));
+    for (int i = 0; i < n; ++i) {
+      ftgcr_handle* h = hs_all[id[i]];
+      const BeginArgs b = begin_args(h, rhs[id[i]], x[id[i]], x[id[i]], plans ? plans[id[i]] : nullptr);
+      k_begin_solve<T><<<1, 64, 0, st>>>((SolveDev<T>*)h->sdev, b, d_act, n, i, 0, i == 0 ? d_ctl : nullptr);
+      CK(cudaGetLastError());
+    }
+    const int max_rounds = (int)std::min<long long>(1 << 30, 2 * max_steps + 8 * ((long long)max_outer + 2) + 16);
+    rc = band ? launch_band<T>(kb, (SolveDev<T>* const*)d_solves, d_act, d_cta, d_nt, d_cnt, d_ctl, d_diag, max_rounds,
+                               grid, smem, st)
+              : launch_persistent<T>(kb, (SolveDev<T>* const*)d_solves, d_nt, d_act, n, d_ctl, d_diag, max_rounds, grid,
+                                     smem, split, st);
+    if (rc) {
+      cudaFreeAsync(buf, st);
+      return rc;
+    }
+    for (int i : id) {
+      ftgcr_handle* h = hs_all[i];
+      CK(cudaMemcpyAsync(h->h_result, h->result, sizeof(SolveState), cudaMemcpyDeviceToHost, st));
+      CK(cudaMemcpyAsync(h->h_ctl, d_ctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
+      h->last_stream = st;
+      h->solved = 1;
+    }
+    CK(cudaFreeAsync(buf, st));
   }
-  CK(cudaMemsetAsync(d_act, 0, sizeof(int) * 2 * n, st));
-  for (int i = 0; i < n; ++i) {
-    const BeginArgs b = begin_args(hs[i], rhs[i], x[i], x[i], plans ? plans[i] : nullptr);
-    k_begin_solve<T><<<1, 64, 0, st>>>((SolveDev<T>*)hs[i]->sdev, b, d_act, n, i, 0, i == 0 ? d_ctl : nullptr);
-    CK(cudaGetLastError());
-  }
-  const int max_rounds = (int)std::min<long long>(1 << 30, 2 * max_steps + 8 * ((long long)max_outer + 2) + 16);
-  rc = launch_persistent<T>(kb, (SolveDev<T>* const*)d_solves, d_nt, d_act, n, d_ctl, d_diag, max_rounds, grid, smem,
-                            split, st);
-  if (rc) {
-    cudaFreeAsync(buf, st);
-    return rc;
-  }
-  for (int i = 0; i < n; ++i) {
-    CK(cudaMemcpyAsync(hs[i]->h_result, hs[i]->result, sizeof(SolveState), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(hs[i]->h_ctl, d_ctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
-    hs[i]->last_stream = st;
-    hs[i]->solved = 1;
-  }
-  CK(cudaFreeAsync(buf, st));
   return FTGCR_OK;
 }
 
@@ -1278,6 +1528,16 @@ struct SlotTableImpl {
   SolveState* d_results = nullptr;  // [n] result records gathered after a launch
   SolveState* h_results = nullptr;  // pinned: their copy
   int grid_cap = 0;
+  // the banded solves' launch (at most kMaxTeamCtas CTAs, one team each at most)
+  int* d_bact = nullptr;            // [n] running flags
+  unsigned int* d_bcnt = nullptr;   // [kMaxTeamCtas] barrier counters, 128 bytes apart
+  LaunchCtl* d_bctl = nullptr;
+  TeamCta* d_bcta = nullptr;        // schedule, and its pinned host copy
+  int* d_border = nullptr;
+  TeamCta* h_bcta = nullptr;
+  int* h_border = nullptr;
+  int* h_bact = nullptr;            // pinned: read back after a launch
+  LaunchCtl* h_bctl = nullptr;
   std::vector<ftgcr_handle*> slot;
   std::vector<char> launched;  // slots occupied when the last launch was enqueued
 };
@@ -1302,37 +1562,74 @@ __global__ void k_gather_results(SolveDev<T>* const* solves, SlotMask mask, int 
 
 template <typename T>
 int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
-  int kb = 4;
-  size_t smem = 1;
-  long long tiles = 0;
-  int split = 0;
-  for (ftgcr_handle* h : t->slot)
-    if (h) {
+  bool any = false;
+  for (int s = 0; s < t->n; ++s) {
+    t->launched[s] = t->slot[s] != nullptr;
+    any = any || t->launched[s];
+  }
+  if (!any) return FTGCR_OK;
+  t->h_ctl_out->err = 0;
+  t->h_ctl_out->round_end = t->round;
+  t->h_bctl->err = 0;
+  for (int band = 0; band < 2; ++band) {
+    int kb = 4;
+    size_t smem = 1;
+    long long tiles = 0;
+    int split = 0;
+    std::vector<int> id;
+    for (int s = 0; s < t->n; ++s) {
+      const ftgcr_handle* h = t->slot[s];
+      if (!h || (h->wide == kWideBand) != (band == 1)) continue;
+      id.push_back(s);
       split = std::max(split, h->wide);
       kb = std::max(kb, kbound(h->k));
       smem = std::max(smem, h->smem);
       tiles += h->nt;
     }
-  if (tiles == 0) return FTGCR_OK;
-  int rc = configure_kernel<T>(kb, split, smem);
-  if (rc) return rc;
-  int occ = 0;
-  rc = occupancy<T>(kb, split, smem, &occ);
-  if (rc) return rc;
-  if (occ < 1) return FTGCR_ERR_ARG;
-  const int grid = (int)std::min<long long>({tiles, (long long)device_info(t->dev).sms * occ, (long long)t->grid_cap});
-  for (int s = 0; s < t->n; ++s) t->launched[s] = t->slot[s] != nullptr;
-  t->h_ctl_in->counter = 0;
-  t->h_ctl_in->err = 0;
-  t->h_ctl_in->round0 = t->round;
-  t->h_ctl_in->round_end = t->round;
-  t->h_ctl_in->nonfinite = 0;
-  CK(cudaMemcpyAsync(t->d_ctl, t->h_ctl_in, sizeof(LaunchCtl), cudaMemcpyHostToDevice, st));
-  rc = launch_persistent<T>(kb, (SolveDev<T>* const*)t->d_solves, t->d_nt, t->d_act, t->n, t->d_ctl, t->d_diag,
-                            max_rounds, grid, smem, split, st);
-  if (rc) return rc;
-  CK(cudaMemcpyAsync(t->h_ctl_out, t->d_ctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(t->h_act, t->d_act, sizeof(int) * 2 * t->n, cudaMemcpyDeviceToHost, st));
+    if (id.empty()) continue;
+    int rc = configure_kernel<T>(kb, split, smem);
+    if (rc) return rc;
+    int occ = 0;
+    rc = occupancy<T>(kb, split, smem, &occ);
+    if (rc) return rc;
+    if (occ < 1) return FTGCR_ERR_ARG;
+    if (band) {
+      std::vector<long long> points;
+      std::vector<int> nts;
+      for (int s : id) {
+        points.push_back(t->slot[s]->N);
+        nts.push_back(t->slot[s]->nt);
+      }
+      TeamPlan tp;
+      plan_teams(points, nts, std::min(device_info(t->dev).sms, kMaxTeamCtas), &tp);
+      const int grid = (int)tp.cta.size();
+      // the previous launch, whose copies read these, has been collected
+      for (int i = 0; i < grid; ++i) t->h_bcta[i] = tp.cta[i];
+      for (size_t i = 0; i < tp.order.size(); ++i) t->h_border[i] = id[tp.order[i]];
+      CK(cudaMemcpyAsync(t->d_bcta, t->h_bcta, sizeof(TeamCta) * grid, cudaMemcpyHostToDevice, st));
+      CK(cudaMemcpyAsync(t->d_border, t->h_border, sizeof(int) * tp.order.size(), cudaMemcpyHostToDevice, st));
+      CK(cudaMemsetAsync(t->d_bcnt, 0, 128 * (size_t)tp.teams, st));
+      CK(cudaMemsetAsync(t->d_bctl, 0, sizeof(LaunchCtl), st));
+      rc = launch_band<T>(kb, (SolveDev<T>* const*)t->d_solves, t->d_bact, t->d_bcta, t->d_border, t->d_bcnt, t->d_bctl,
+                          t->d_diag, max_rounds, grid, smem, st);
+      if (rc) return rc;
+      CK(cudaMemcpyAsync(t->h_bctl, t->d_bctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
+      CK(cudaMemcpyAsync(t->h_bact, t->d_bact, sizeof(int) * t->n, cudaMemcpyDeviceToHost, st));
+      continue;
+    }
+    const int grid = (int)std::min<long long>({tiles, (long long)device_info(t->dev).sms * occ, (long long)t->grid_cap});
+    t->h_ctl_in->counter = 0;
+    t->h_ctl_in->err = 0;
+    t->h_ctl_in->round0 = t->round;
+    t->h_ctl_in->round_end = t->round;
+    t->h_ctl_in->nonfinite = 0;
+    CK(cudaMemcpyAsync(t->d_ctl, t->h_ctl_in, sizeof(LaunchCtl), cudaMemcpyHostToDevice, st));
+    rc = launch_persistent<T>(kb, (SolveDev<T>* const*)t->d_solves, t->d_nt, t->d_act, t->n, t->d_ctl, t->d_diag,
+                              max_rounds, grid, smem, split, st);
+    if (rc) return rc;
+    CK(cudaMemcpyAsync(t->h_ctl_out, t->d_ctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(t->h_act, t->d_act, sizeof(int) * 2 * t->n, cudaMemcpyDeviceToHost, st));
+  }
   SlotMask mask;
   memset(&mask, 0, sizeof mask);
   for (int s = 0; s < t->n; ++s)
@@ -1439,6 +1736,39 @@ static void fill_handle_params(ftgcr_handle* h, const ftgcr_grid* g, int32_t k, 
   }
   h->plan = smem_plan(h->nlon, h->nlat, h->nt, mixed, elem, h->precond, h->split, (size_t)smem_limit, gconsts);
   h->wide = h->split || h->plan.gconsts;
+  // banded rounds where the line preconditioner runs in one pass: the bands
+  // the SM count gives (or asked for), thinner only where a band's rows do not
+  // fit on chip
+  if (h->precond != FTGCR_PRECOND_LINE || h->noalloc || (h->flags & (FTGCR_FLAG_ORACLE_ORDER | FTGCR_FLAG_SPLIT_ROUNDS)))
+    return;
+  const int hpar = (h->nlat + sms - 1) / sms;
+  int nt = g->tiles > 0 ? std::min(g->tiles, h->nlat) : (h->nlat + hpar - 1) / hpar;
+  bool fits = band_layout(h->nlon, h->nlat, nt, mixed, k, (size_t)(smem_limit + kStaticSmemReserve - kBandFixed), &h->bl);
+  while (!fits && g->tiles == 0 && nt < h->nlat) {
+    nt = std::min(h->nlat, nt + sms);
+    fits = band_layout(h->nlon, h->nlat, nt, mixed, k, (size_t)(smem_limit + kStaticSmemReserve - kBandFixed), &h->bl);
+  }
+  if (!fits) return;
+  // Where neighbours must exchange edge rows of e, mixed one-pass rounds (which
+  // form e on the halo rows themselves) with a CTA per band stay ahead for two
+  // kinds of bands (with several bands a CTA never: 2048 x 1024 4.23 / 3.43):
+  // large ones, whose vectors and face coefficients the banded kernel mostly
+  // reads from L2 (one-pass against banded, k = 4, ms: 1440 x 721 of 1800
+  // groups a band 1.70 / 1.78, 1200 x 760 of 1500 1.54 / 1.56; but 1400 x 600
+  // of 1400 1.53 / 1.41, 1024 x 750 of 1280 1.36 / 1.28; even for k > 4, 1440 x
+  // 721, k = 5: 2.07 / 2.05), and k <= 2, where
+  // their own pass over the directions is short (1208 x 531, k = 2: 1.22 /
+  // 1.24; k = 4 is ahead when banded).  Widths off the 16-byte unit are always
+  // ahead when banded (1209 x 531: 3.00 / 1.62, 801 x 401: 1.78 / 1.04).
+  if (mixed && !h->split && !gconsts && h->plan.bytes <= (size_t)smem_limit && h->nt <= sms && !h->bl.local &&
+      g->nlon % 4 == 0 && k <= 4) {
+    const int groups = (h->nlat + nt - 1) / nt * (g->nlon / 4);
+    if (groups > kOnePassGroups || k <= 2) return;
+  }
+  h->nt = nt;
+  h->split = 0;
+  h->wide = kWideBand;
+  h->plan.bytes = 0;  // fits: bl.bytes is what the launch takes
 }
 
 int ftgcr_create(const ftgcr_grid* grid, const ftgcr_coeffs* coeffs, int32_t k, double tol, ftgcr_handle** out) {
@@ -1685,8 +2015,11 @@ int table_create(int precision, int max_slots, SlotTable** out) {
   t->grid_cap = di.sms * 4;
   const size_t b_solves = align256(sizeof(void*) * max_slots), b_nt = align256(sizeof(int) * max_slots),
                b_act = align256(sizeof(int) * 2 * max_slots), b_ctl = align256(sizeof(LaunchCtl)),
-               b_diag = align256(sizeof(int) * 4 * t->grid_cap), b_res = align256(sizeof(SolveState) * max_slots);
-  const size_t total = b_solves + b_nt + b_act + b_ctl + b_diag + b_res;
+               b_diag = align256(sizeof(int) * 4 * t->grid_cap), b_res = align256(sizeof(SolveState) * max_slots),
+               b_bact = align256(sizeof(int) * max_slots), b_bcnt = align256(128 * (size_t)kMaxTeamCtas),
+               b_bcta = align256(sizeof(TeamCta) * kMaxTeamCtas);
+  const size_t legacy = b_solves + b_nt + b_act + b_ctl + b_diag + b_res;
+  const size_t total = legacy + 2 * b_bact + b_bcnt + b_ctl + b_bcta;
   if (cudaMalloc(&t->buf, total) != cudaSuccess) {
     cudaGetLastError();
     delete t;
@@ -1698,7 +2031,16 @@ int table_create(int precision, int max_slots, SlotTable** out) {
   t->d_ctl = (LaunchCtl*)(t->buf + b_solves + b_nt + b_act);
   t->d_diag = (int*)(t->buf + b_solves + b_nt + b_act + b_ctl);
   t->d_results = (SolveState*)(t->buf + b_solves + b_nt + b_act + b_ctl + b_diag);
+  t->d_bact = (int*)(t->buf + legacy);
+  t->d_border = (int*)(t->buf + legacy + b_bact);
+  t->d_bcnt = (unsigned int*)(t->buf + legacy + 2 * b_bact);
+  t->d_bctl = (LaunchCtl*)(t->buf + legacy + 2 * b_bact + b_bcnt);
+  t->d_bcta = (TeamCta*)(t->buf + legacy + 2 * b_bact + b_bcnt + b_ctl);
   int rc = cuda_status(cudaMemset(t->buf, 0, total));
+  if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bcta, sizeof(TeamCta) * kMaxTeamCtas));
+  if (!rc) rc = cuda_status(cudaMallocHost(&t->h_border, sizeof(int) * max_slots));
+  if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bact, sizeof(int) * max_slots));
+  if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bctl, sizeof(LaunchCtl)));
   if (!rc) rc = cuda_status(cudaMallocHost(&t->h_ctl_in, sizeof(LaunchCtl)));
   if (!rc) rc = cuda_status(cudaMallocHost(&t->h_ctl_out, sizeof(LaunchCtl)));
   if (!rc) rc = cuda_status(cudaMallocHost(&t->h_act, sizeof(int) * 2 * max_slots));
@@ -1714,6 +2056,10 @@ int table_create(int precision, int max_slots, SlotTable** out) {
 void table_destroy(SlotTable* t) {
   if (!t) return;
   if (t->buf) cudaFree(t->buf);
+  if (t->h_bcta) cudaFreeHost(t->h_bcta);
+  if (t->h_border) cudaFreeHost(t->h_border);
+  if (t->h_bact) cudaFreeHost(t->h_bact);
+  if (t->h_bctl) cudaFreeHost(t->h_bctl);
   if (t->h_ctl_in) cudaFreeHost(t->h_ctl_in);
   if (t->h_ctl_out) cudaFreeHost(t->h_ctl_out);
   if (t->h_act) cudaFreeHost(t->h_act);
@@ -1736,7 +2082,8 @@ int table_begin(SlotTable* t, int slot, ftgcr_handle* h, const double* rhs, doub
   if (rc) return rc;
   // written by a kernel, not copied from pageable host memory: such a copy
   // may wait for the launch still running on the stream
-  k_table_place<<<1, 1, 0, st>>>(t->d_solves, t->d_nt, slot, h->sdev, h->nt);
+  const bool band = h->wide == kWideBand;  // not in the other kernels' launch: no tiles there
+  k_table_place<<<1, 1, 0, st>>>(t->d_solves, t->d_nt, slot, h->sdev, band ? 0 : h->nt);
   CK(cudaGetLastError());
   if (check) {  // the handle's own control block carries the flag
     const int cg = (int)std::min<long long>((h->N + 255) / 256, 1024);
@@ -1747,10 +2094,12 @@ int table_begin(SlotTable* t, int slot, ftgcr_handle* h, const double* rhs, doub
   const BeginArgs b = begin_args(h, rhs, x, x, plan);
   // parity -1: the begin may be enqueued behind a launch still running
   const LaunchCtl* chk = check ? h->ctl : nullptr;
+  int* act = band ? t->d_bact : t->d_act;
+  const int nact = band ? 0 : t->n;  // banded solves: one flag a slot, whatever the parity
   if (t->precision == FTGCR_MIXED)
-    k_begin_solve<float><<<1, 64, 0, st>>>((SolveDev<float>*)h->sdev, b, t->d_act, t->n, slot, -1, nullptr, chk);
+    k_begin_solve<float><<<1, 64, 0, st>>>((SolveDev<float>*)h->sdev, b, act, nact, slot, -1, nullptr, chk);
   else
-    k_begin_solve<double><<<1, 64, 0, st>>>((SolveDev<double>*)h->sdev, b, t->d_act, t->n, slot, -1, nullptr, chk);
+    k_begin_solve<double><<<1, 64, 0, st>>>((SolveDev<double>*)h->sdev, b, act, nact, slot, -1, nullptr, chk);
   CK(cudaGetLastError());
   t->slot[slot] = h;
   return FTGCR_OK;
@@ -1769,16 +2118,17 @@ int table_collect(SlotTable* t, cudaStream_t st, int* finished) {
   for (int s = 0; s < t->n; ++s) any = any || (t->launched[s] && t->slot[s]);
   if (!any) return FTGCR_OK;
   CK(cudaStreamSynchronize(st));
-  const int err = t->h_ctl_out->err;
+  const int err = t->h_ctl_out->err ? t->h_ctl_out->err : t->h_bctl->err;
   t->round = t->h_ctl_out->round_end;
   const int par = (int)(t->round & 1);
   for (int s = 0; s < t->n; ++s) {
     ftgcr_handle* h = t->slot[s];
     if (!h || !t->launched[s]) continue;  // begun after the launch: runs in the next one
     t->launched[s] = 0;
-    if (!err && t->h_act[par * t->n + s]) continue;
+    const bool band = h->wide == kWideBand;
+    if (!err && (band ? t->h_bact[s] : t->h_act[par * t->n + s])) continue;
     memcpy(h->h_result, t->h_results + s, sizeof(SolveState));  // gathered after the launch
-    *h->h_ctl = *t->h_ctl_out;
+    *h->h_ctl = band ? *t->h_bctl : *t->h_ctl_out;
     h->last_stream = st;
     h->solved = 1;
     h->last_status = err ? FTGCR_ERR_TIMEOUT : status_from_result(h);
@@ -1789,6 +2139,7 @@ int table_collect(SlotTable* t, cudaStream_t st, int* finished) {
     // the launch is abandoned: its solves' state is not resumable, and the
     // next launch starts from a clean table
     CK(cudaMemsetAsync(t->d_act, 0, sizeof(int) * 2 * t->n, st));
+    CK(cudaMemsetAsync(t->d_bact, 0, sizeof(int) * t->n, st));
     CK(cudaStreamSynchronize(st));
     return FTGCR_ERR_TIMEOUT;
   }
@@ -1798,6 +2149,7 @@ int table_collect(SlotTable* t, cudaStream_t st, int* finished) {
 void table_abandon(SlotTable* t, cudaStream_t st) {
   for (auto& h : t->slot) h = nullptr;
   cudaMemsetAsync(t->d_act, 0, sizeof(int) * 2 * t->n, st);
+  cudaMemsetAsync(t->d_bact, 0, sizeof(int) * t->n, st);
   cudaStreamSynchronize(st);
 }
 

@@ -1,0 +1,10 @@
+// Banded-round kernel instances for at most 4 Krylov directions.
+#define FTGCR_THREADS 512
+#include "ftgcr_instances.h"
+#include "ftgcr_band.cuh"
+
+namespace ftgcr {
+const void* band_kernel_k4(bool fp64) {
+  return fp64 ? (const void*)k_ftgcr_band<double, 4> : (const void*)k_ftgcr_band<float, 4>;
+}
+}  // namespace ftgcr

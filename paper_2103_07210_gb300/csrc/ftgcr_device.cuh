@@ -19,7 +19,10 @@ constexpr int kMaxFaults = 64;
 constexpr int kMaxDetect = 16;
 constexpr int kNPart = kMaxK + 4;      // partial sums per tile (each a double-double pair)
 constexpr int kPartStride = 2 * kNPart;  // doubles per tile in the partials buffer
-constexpr int kThreads = 256;
+#ifndef FTGCR_THREADS
+#define FTGCR_THREADS 256
+#endif
+constexpr int kThreads = FTGCR_THREADS;  // of the persistent kernels in this translation unit
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned long long kBarrierTimeoutNs = 2000000000ull;  // 2 s
 constexpr unsigned long long kKernelTimeoutNs = 60000000000ull;  // 60 s
@@ -96,6 +99,7 @@ struct SolveState {
   int ndetect;
   int ecur;  // buffer of e, L(e) written by the latest PA / PF
   int refused;  // the solve did not start: a staged host input was not finite
+  long long round;  // banded rounds: rounds run so far (its parity picks the partial-sum buffer)
   long long detect_step[kMaxDetect];
   double detect_ratio[kMaxDetect];
 };
@@ -173,6 +177,20 @@ struct SolveDev {
   // (wide rows, where staging them would leave bands thinner than the SM
   // count gives)
   int cs_global;
+  // banded rounds (ftgcr_band.cuh; local: halo rows formed, not received, in a
+  // CTA with one band): the layout of a row in shared memory (Q
+  // planes of NP 16-byte units, pieces of Q units, NPc pieces in use, solved
+  // by 2^lG warps), the pitch PC of a plane of the line-solve constants, the
+  // bytes of a row, of a row's constants and of a band's vector, where the
+  // threads' sums, the constants (cs_staged), the face coefficients (ts_staged)
+  // and the nbuf vector buffers sit in shared memory
+  int band, local, lq, NP, NPc, lG, PC, nbuf, cs_staged, ts_staged;
+  int rowb, conb, bufb, faceb, red_off, con_off, ts_off, buf_off;
+  int NG, rb, rx;  // groups of four columns in a row; rows of a band: rb, one more in the first rx bands
+  int mega;        // bands a CTA with several takes at a time
+  float rng;       // 1 / NG
+  unsigned int solve_id;        // counts the handle's solves
+  uint4* hrow;                  // [2][nt][2] the bands' first and last rows of e (local: L(e)) as packets
 };
 
 // --------------------------------------------------------------- helpers
@@ -214,9 +232,8 @@ __device__ __forceinline__ DD dd_add(DD a, DD b) {
 // differs from Dot2's by about the rounding of a few hundred terms (relative
 // 1e-14 at most), far below the margins of the fault test.  FP32 vectors: the
 // product of two floats is exact as a float pair (TwoProduct with fmaf) and is
-// accumulated in a float-float pair; warps combine float-float pairs in FP32
-// and only per-warp sums reach FP64 (GB300's FP64 pipe is ~60x slower than
-// FP32).
+// accumulated in a float-float pair (GB300's FP64 pipe is ~60x slower than
+// FP32).  Above the thread every sum runs in fixed point (Fx below).
 template <typename T>
 struct Acc;
 template <>
@@ -250,12 +267,6 @@ struct AccF64 {
   double s;
   __device__ __forceinline__ AccF64() : s(0.0) {}
   __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ __forceinline__ DD warp_sum() const {
-    double v = s;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return DD{v, 0.0};
-  }
 };
 template <>
 struct Acc<float> {
@@ -271,26 +282,12 @@ struct Acc<float> {
     hi = s;
     lo = lo + (err + pe);
   }
-  __device__ __forceinline__ DD warp_sum() const {
-    float h = hi, l = lo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float h2 = __shfl_xor_sync(0xffffffffu, h, o);
-      const float l2 = __shfl_xor_sync(0xffffffffu, l, o);
-      const float t = h + h2;
-      const float z = t - h;
-      const float q = (h - (t - z)) + (h2 - z);
-      h = t;
-      l = (l + l2) + q;
-    }
-    return DD{(double)h, (double)l};
-  }
 };
 
-// Sums of doubles across threads in fixed point (FP64 path).  GB300 issues an
-// FP64 warp instruction every 18 cycles per SM whatever the active lanes, so a
-// double-double tree over a CTA (8 warps x 5 levels x 8 operations a value)
-// took 11 us of a 28 us step round on a 64 x 32 grid.  The integer pipe is some 70 times
+// Sums across threads in fixed point.  GB300 issues an FP64 warp instruction
+// every 18 cycles per SM whatever the active lanes, so a double-double tree
+// over a CTA (8 warps x 5 levels x 8 operations a value) took 11 us of a
+// 28 us step round on a 64 x 32 grid.  The integer pipe is some 70 times
 // wider: each double's 53-bit mantissa is placed in a 128-bit two's-complement
 // integer whose unit is fixed by the largest exponent among the terms (bits
 // 64..116 hold the largest term, 10 bits above it take the carries of up to
@@ -323,24 +320,6 @@ __device__ __forceinline__ void fx_add(Fx& v, double x, int E) {
   }
   v.lo += l;
   v.hi += (long long)(h + (v.lo < l ? 1ull : 0ull));
-}
-// a += b, both brought to the larger exponent.
-__device__ __forceinline__ void fx_merge(Fx& a, Fx b) {
-  const int E = a.e > b.e ? a.e : b.e;
-  auto down = [&](Fx& x) {
-    const int sh = E - x.e;
-    if (sh == 0) return;
-    if (sh < 64)
-      x.lo = (x.lo >> sh) | (((unsigned long long)x.hi << 1) << (63 - sh));
-    else
-      x.lo = (unsigned long long)(x.hi >> (sh < 127 ? sh - 64 : 63));
-    x.hi = sh < 64 ? x.hi >> sh : x.hi >> 63;
-    x.e = E;
-  };
-  down(a);
-  down(b);
-  a.lo += b.lo;
-  a.hi += b.hi + (a.lo < b.lo ? 1ll : 0ll);
 }
 // Sum over the warp, the same in every lane: five integer reductions of
 // 26-bit pieces (32 of which add up within 32 bits).  Every lane's v.e alike.
@@ -380,56 +359,132 @@ __device__ __forceinline__ DD fx_dd(const Fx& v) {
   return DD{scale(d1, v.e - 1075), scale(d2, v.e - 1075 - 50)};
 }
 
-// Per-CTA partial sums: each warp contributes its sum of every value, the CTA
-// combines the warps' and writes nv pairs.  FP64 path: fixed point (above),
-// one double-double written.  FP32 path: each warp's pair is first rounded to
-// one double, then plain FP64 adds in a fixed binary tree (depth 3 for 8
-// warps: GB300's FP64 latency makes a serial chain expensive).
-struct CtaRed {
-  union {
-    DD w[kWarps][kNPart];
-    Fx f[kWarps][kNPart];
-  };
-};
-__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, DD x) {
-  if ((threadIdx.x & 31) == 0) cr.w[threadIdx.x >> 5][v] = x;
+// The value rounded to one double: the leading 64 bits, normalised so that
+// cancellation loses none of the 53 kept.
+__device__ __forceinline__ double fx_double(const Fx& v) {
+  if (v.e >= kFxNaN) return __longlong_as_double(0x7ff8000000000000ll);
+  const unsigned long long h = (unsigned long long)(v.hi ^ (v.hi >> 63));  // leading zeros of the magnitude
+  long long t;
+  int e = v.e - 1075;
+  if (h) {
+    const int sh = __clzll((long long)h) - 1;
+    t = sh ? (long long)(((unsigned long long)v.hi << sh) | (v.lo >> (64 - sh))) : v.hi;
+    e -= sh;
+  } else if (((long long)v.lo >> 63) == v.hi) {  // the low word with its sign
+    t = (long long)v.lo;
+    e -= 64;
+  } else {
+    t = (long long)(((unsigned long long)v.hi << 62) | (v.lo >> 2));
+    e -= 62;
+  }
+  const double d = __ll2double_rn(t);
+  const int a = e / 2, b = e - a;
+  return (d * __longlong_as_double((long long)(1023 + a) << 52)) * __longlong_as_double((long long)(1023 + b) << 52);
 }
-__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const Acc<float>& a) { cta_red_put(cr, v, a.warp_sum()); }
-__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const AccF64& a) { cta_red_put(cr, v, a.warp_sum()); }
-__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const Acc<double>& a) {
-  int E = fx_exp(a.p);
-  if (a.ex) E = max(E, fx_exp(a.s));
-  E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
+
+// Per-CTA partial sums: each warp contributes its sum of every value, then one
+// warp per value combines them.  These, like everything a round runs once, are
+// kept small and out of line: a round that touches few points is bound by
+// instruction fetch (with all of it inlined, 64 x 32 rounds took 19 us for
+// under 1 us of arithmetic).
+struct CtaRed {
+  Fx f[kWarps][kNPart];
+  int stride;  // doubles from one value of a band's partial sums to the next
+};
+// Brings x to exponent E >= x.e.
+__device__ __forceinline__ void fx_down(Fx& x, int E) {
+  const int sh = E - x.e;
+  if (sh >= 64) {
+    x.lo = (unsigned long long)(x.hi >> min(sh - 64, 63));
+    x.hi = x.hi >> 63;
+  } else if (sh > 0) {
+    x.lo = (x.lo >> sh) | (((unsigned long long)x.hi << 1) << (63 - sh));
+    x.hi = x.hi >> sh;
+  }
+  x.e = E;
+}
+// Warp sum of p (and of s, the smaller part of a compensated sum) into slot v.
+static __device__ __noinline__ void red_put_d(CtaRed& cr, int v, double p, double s) {
+  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(fx_exp(p), fx_exp(s)));
   Fx x{0ull, 0ll, E < 0x7ff ? E : kFxNaN};
   if (E < 0x7ff) {
-    fx_add(x, a.p, E);
-    if (a.ex) fx_add(x, a.s, E);
+    const double t[2] = {p, s};
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      const double y = q ? t[1] : t[0];
+      if (q == 0 || s != 0.0) fx_add(x, y, E);
+    }
     x = fx_warp_sum(x);
   }
   if ((threadIdx.x & 31) == 0) cr.f[threadIdx.x >> 5][v] = x;
 }
-template <typename T>
-__device__ __forceinline__ void cta_red_finish(CtaRed& cr, int nv, double* out, int v0 = 0) {
+// A float-float pair over the warp: 64-bit integers with the largest term's
+// mantissa in bits 33..56 (terms cut below 2^-57 of it; float-float adds err by
+// 2^-48), summed as three integer reductions.  *E: biased exponent of the unit,
+// value = sum 2^(E - 183); 0xff: not finite.
+__device__ __forceinline__ long long fx_float(float hi, float lo, int* E) {
+  auto ex = [](float x) {
+    const int e = (int)(__float_as_uint(x) >> 23) & 0xff;
+    return e > 0 ? e : 1;
+  };
+  const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(ex(hi), ex(lo)));
+  auto fix = [&](float x) {
+    const unsigned u = __float_as_uint(x);
+    const unsigned f = (u & 0x7fffffu) | ((u & 0x7f800000u) ? 0x800000u : 0u);
+    const int sh = m - ex(x);
+    const long long q = sh < 58 ? (long long)(((unsigned long long)f << 33) >> sh) : 0ll;
+    return (int)u < 0 ? -q : q;
+  };
+  const unsigned long long t = (unsigned long long)(fix(hi) + fix(lo));
+  constexpr unsigned M = (1u << 22) - 1u;
+  const unsigned long long s0 = __reduce_add_sync(0xffffffffu, (unsigned)t & M),
+                           s1 = __reduce_add_sync(0xffffffffu, (unsigned)(t >> 22) & M),
+                           s2 = __reduce_add_sync(0xffffffffu, (unsigned)(t >> 44));
+  *E = m;
+  return (long long)(s0 + (s1 << 22) + (s2 << 44));
+}
+__device__ __forceinline__ double fx_float_sum(float hi, float lo) {
+  int E;
+  const long long sum = fx_float(hi, lo, &E);
+  if (E == 0xff) return __longlong_as_double(0x7ff8000000000000ll);
+  return __ll2double_rn(sum) * __longlong_as_double((long long)(1023 + E - 183) << 52);
+}
+static __device__ __noinline__ void red_put_f(CtaRed& cr, int v, float hi, float lo) {
+  int E;
+  const long long sum = fx_float(hi, lo, &E);
+  // four bits of room for the other warps' sums
+  Fx x{(unsigned long long)sum << 60, sum >> 4, E + 896};
+  if (E == 0xff) x.e = kFxNaN;
+  if ((threadIdx.x & 31) == 0) cr.f[threadIdx.x >> 5][v] = x;
+}
+__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const Acc<double>& a) {
+  red_put_d(cr, v, a.p, a.ex ? a.s : 0.0);
+}
+__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const AccF64& a) { red_put_d(cr, v, a.s, 0.0); }
+__device__ __forceinline__ void cta_red_put(CtaRed& cr, int v, const Acc<float>& a) { red_put_f(cr, v, a.hi, a.lo); }
+__device__ __forceinline__ void cta_red_zero(CtaRed& cr, int v) {
+  if ((threadIdx.x & 31) == 0) cr.f[threadIdx.x >> 5][v] = Fx{0ull, 0ll, 1};
+}
+// Value v of the whole CTA, the same in every lane (one warp, after a block
+// barrier).
+__device__ __forceinline__ DD cta_red_value(const CtaRed& cr, int v) {
+  const int lane = threadIdx.x & 31;
+  Fx x{0ull, 0ll, 1};
+  if (lane < kWarps) x = cr.f[lane][v];
+  fx_down(x, (int)__reduce_max_sync(0xffffffffu, (unsigned)x.e));
+  return fx_dd(fx_warp_sum(x));
+}
+// Values [v0, nv) of the CTA written to `out` (add: added to what is there).
+static __device__ __noinline__ void cta_red_finish(CtaRed& cr, int nv, double* out, int v0 = 0, bool add = false) {
   __syncthreads();
-  if (threadIdx.x >= v0 && threadIdx.x < nv) {
-    const int v = threadIdx.x;
-    if constexpr (sizeof(T) == 8) {
-      Fx t = cr.f[0][v];
-#pragma unroll
-      for (int w = 1; w < kWarps; ++w) fx_merge(t, cr.f[w][v]);
-      const DD d = fx_dd(t);
-      out[2 * v] = d.hi;
-      out[2 * v + 1] = d.lo;
-    } else {
-      double t[kWarps];
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) t[w] = cr.w[w][v].hi + cr.w[w][v].lo;
-#pragma unroll
-      for (int h = 1; h < kWarps; h <<= 1)
-#pragma unroll
-        for (int w = 0; w + h < kWarps; w += 2 * h) t[w] = t[w] + t[w + h];
-      out[2 * v] = t[0];
-      out[2 * v + 1] = 0.0;
+#pragma unroll 1
+  for (int v = v0 + (int)(threadIdx.x >> 5); v < nv; v += kWarps) {
+    DD d = cta_red_value(cr, v);
+    if ((threadIdx.x & 31) == 0) {
+      double* o = out + (long long)v * cr.stride;
+      if (add) d = dd_add(DD{o[0], o[1]}, d);
+      o[0] = d.hi;
+      o[1] = d.lo;
     }
   }
 }
@@ -492,26 +547,46 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 // Grid barrier for a cooperative launch: monotonic arrival counter (zeroed
 // before the launch), bounded spin.  On timeout the CTA raises *err and
 // returns; every CTA checks *err after each barrier, so the kernel ends
-// within one more timeout.  Returns false when the kernel must stop.
-__device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int target, int* err, int* bail_smem) {
+// within one more timeout.  Returns false when the kernel must stop.  While
+// thread 0 waits, the other warps run `meanwhile` (called by every thread of
+// warps 1 and up).
+__device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int* p) {
+  unsigned int v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+template <typename F>
+__device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int target, int* err, int* bail_smem,
+                                             F&& meanwhile) {
   __syncthreads();
   if (threadIdx.x == 0) {
     // arrive with release semantics (the block's writes, ordered before by the
-    // block barrier, become visible with the count), wait with acquire loads
+    // block barrier, become visible with the count); wait with relaxed loads
+    // and one acquire fence after them
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(1u) : "memory");
-    unsigned long long t0 = globaltimer();
+    unsigned long long t0 = 0ull;
     unsigned int it = 0;
-    while (ld_acquire_u32(counter) < target) {
-      if ((++it & 63u) == 0u && globaltimer() - t0 > kBarrierTimeoutNs) {
-        atomicExch(err, 1);
-        break;
+    while (ld_relaxed_u32(counter) < target) {
+      if ((++it & 63u) == 0u) {
+        const unsigned long long t = globaltimer();
+        if (t0 == 0ull) t0 = t;
+        if (t - t0 > kBarrierTimeoutNs) {
+          atomicExch(err, 1);
+          break;
+        }
       }
-      __nanosleep(20);
     }
-    *bail_smem = ld_acquire_u32(reinterpret_cast<const unsigned int*>(err));
+    const int bad = (int)ld_relaxed_u32(reinterpret_cast<const unsigned int*>(err));
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    *bail_smem = bad;
+  } else if (threadIdx.x >= 32) {
+    meanwhile();
   }
   __syncthreads();
   return *bail_smem == 0;
+}
+__device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int target, int* err, int* bail_smem) {
+  return grid_barrier(counter, target, err, bail_smem, [] {});
 }
 
 // --------------------------------------------------------------- operator

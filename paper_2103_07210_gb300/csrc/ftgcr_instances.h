@@ -15,10 +15,22 @@ const void* persistent_kernel_k16_wide64();
 const void* persistent_kernel_k4_stream();
 const void* persistent_kernel_k8_stream();
 const void* persistent_kernel_k16_stream();
+const void* band_kernel_k4(bool fp64);
+const void* band_kernel_k8(bool fp64);
+const void* band_kernel_k16(bool fp64);
+constexpr int kWideBand = 3;      // banded rounds (ftgcr_band.cuh)
+constexpr int kBandThreads = 512; // their CTAs
+constexpr int kBandFixed = 17 * 1024;  // bytes of their records in shared memory
 // wide 1: the instance for wide-row solves (mixed path: split rounds; FP64
 // path: line-solve factors read from global memory); wide 2 (mixed path): the
-// split-round instance with the streamed step rounds
+// split-round instance with the streamed step rounds; wide kWideBand: banded
+// rounds
 inline const void* persistent_kernel_ptr(int kb, bool fp64, int wide) {
+  if (wide == kWideBand) {
+    if (kb == 4) return band_kernel_k4(fp64);
+    if (kb == 8) return band_kernel_k8(fp64);
+    return band_kernel_k16(fp64);
+  }
   if (wide == 2 && !fp64) {
     if (kb == 4) return persistent_kernel_k4_stream();
     if (kb == 8) return persistent_kernel_k8_stream();

@@ -114,8 +114,11 @@ __device__ int collect_flips(const SolveDev<T>& sd, long long step, unsigned vma
   return n;
 }
 
+// (out of line: rare, and inlined into every loop it made up most of the
+// kernels' code)
 template <typename T>
-__device__ __forceinline__ T apply_flips(T v, long long g, int vec, int nfl, const FlipEnt* fl) {
+__device__ __noinline__ T apply_flips(T v, long long g, int vec, int nfl, const FlipEnt* fl) {
+#pragma unroll 1
   for (int q = 0; q < nfl; ++q)
     if (fl[q].g == g && fl[q].vec == vec) v = flip_bits(v, fl[q].bit);
   return v;
@@ -124,8 +127,9 @@ __device__ __forceinline__ T apply_flips(T v, long long g, int vec, int nfl, con
 // Clean value of the backup at element g of vector vec while it still
 // carries the initialisation flips (see the INIT phase).
 template <typename T>
-__device__ __forceinline__ T apply_patches(T v, long long g, int vec, int npt, const FlipEnt* pt,
-                                           const double* patchval) {
+__device__ __noinline__ T apply_patches(T v, long long g, int vec, int npt, const FlipEnt* pt,
+                                        const double* patchval) {
+#pragma unroll 1
   for (int q = 0; q < npt; ++q)
     if (pt[q].g == g && pt[q].vec == vec) v = (T)__ldcg(patchval + pt[q].q);
   return v;
@@ -141,6 +145,15 @@ __device__ __forceinline__ int count_faults(const SolveDev<T>& sd, long long ste
 
 constexpr unsigned kStateVecs = (1u << V_X) | (1u << V_R) | (1u << V_P) | (1u << V_AP);
 
+// Whether the plan flips x, r, p or Ap at step t + 1 or at a step whose
+// direction may belong to the Krylov cycle of step t.
+template <typename T>
+__device__ __forceinline__ bool state_flip_near(const SolveDev<T>& sd, long long t) {
+  for (int q = 0; q < sd.nfaults; ++q)
+    if (sd.faults[q].step <= t + 1 && sd.faults[q].step >= t - sd.k && ((kStateVecs >> sd.faults[q].vec) & 1u)) return true;
+  return false;
+}
+
 template <typename T>
 __device__ __forceinline__ int count_losses(const SolveDev<T>& sd, long long step) {
   int c = 0;
@@ -151,87 +164,62 @@ __device__ __forceinline__ int count_losses(const SolveDev<T>& sd, long long ste
 // ------------------------------------------------------------ reductions
 // Deterministic sum over the nt tiles of the partials buffer of the first nv
 // values.  Warp v sums value v: lanes take tiles lane, lane+32, ... (all loads
-// issued first).  FP64 path: fixed point, rounded once (double-double trees
-// here took 6 us of every round); FP32 path: added in tile order, then a fixed
-// xor tree, in plain FP64 (per-tile values are already accurate sums).  Every CTA that works on the
+// issued first), in fixed point, rounded once (double-double trees here took
+// 6 us of every round of the FP64 path).  Every CTA that works on the
 // solve gets bitwise the same numbers.
 // Warps w0..kWarps-1 take part (warp w0 + i sums values i, i + (kWarps - w0),
 // ...); the order within a value is the same whichever warp sums it.
-template <typename T>
-__device__ __forceinline__ void reduce_partials(const double* part, int nt, int nv, double* red, int w0 = 0) {
-  constexpr int B = 8;  // tiles loaded per batch per lane, summed in a binary tree
+static __device__ __noinline__ void reduce_partials(const double* part, int nt, int nv, double* red, int w0 = 0) {
+  constexpr int B = 8;  // tiles loaded per batch per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp < w0) return;
+#pragma unroll 1
   for (int v = warp - w0; v < nv; v += kWarps - w0) {
-    if constexpr (sizeof(T) == 8) {
-      // fixed point (see Fx): the tiles' pairs in batches of 32 B
-      Fx sum{0ull, 0ll, 1};
-      for (int t0 = 0; t0 < nt; t0 += 32 * B) {
-        DD tv[B];
-        int E = 1;
+    // fixed point (see Fx): the tiles' pairs in batches of 32 B
+    Fx sum{0ull, 0ll, 1};
+#pragma unroll 1
+    for (int t0 = 0; t0 < nt; t0 += 32 * B) {
+      V16<double> tv[B];
+      int E = 1;
 #pragma unroll
-        for (int q = 0; q < B; ++q) {
-          tv[q] = DD{0.0, 0.0};
-          const int tau = t0 + lane + 32 * q;
-          if (tau < nt) {
-            const V16<double> d = ldv(part + (long long)tau * kPartStride + 2 * v);
-            tv[q] = DD{d.v[0], d.v[1]};
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < B; ++q) E = max(E, max(fx_exp(tv[q].hi), fx_exp(tv[q].lo)));
-        E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
-        Fx x{0ull, 0ll, E < 0x7ff ? E : kFxNaN};
-        if (E < 0x7ff) {
-#pragma unroll
-          for (int q = 0; q < B; ++q)
-            if (t0 + 32 * q < nt) {
-              fx_add(x, tv[q].hi, E);
-              fx_add(x, tv[q].lo, E);
-            }
-          x = fx_warp_sum(x);
-        }
-        if (nt <= 32 * B) {
-          sum = x;
-        } else {
-          // room for the carries of up to 4096 batches (2^20 tiles): 12 bits
-          if (x.e < kFxNaN) {
-            x.lo = (x.lo >> 12) | ((unsigned long long)x.hi << 52);
-            x.hi >>= 12;
-            x.e += 12;
-          }
-          fx_merge(sum, x);
-        }
+      for (int q = 0; q < B; ++q) {
+        tv[q].v[0] = tv[q].v[1] = 0.0;
+        const int tau = t0 + lane + 32 * q;
+        if (tau < nt) tv[q] = ldv(part + (long long)tau * kPartStride + 2 * v);
       }
-      if (lane == 0) {
-        const DD d = fx_dd(sum);
-        red[v] = d.hi + d.lo;
-      }
-    } else {
-      double acc1 = 0.0;
-      for (int t0 = lane; t0 < nt; t0 += 32 * B) {
-        DD tv[B];
 #pragma unroll
-        for (int q = 0; q < B; ++q) {
-          const int tau = t0 + 32 * q;
-          tv[q] = DD{0.0, 0.0};
-          if (tau < nt) {
-            tv[q].hi = __ldcg(part + (long long)tau * kPartStride + 2 * v);
-            tv[q].lo = __ldcg(part + (long long)tau * kPartStride + 2 * v + 1);
-          }
+      for (int q = 0; q < B; ++q) E = max(E, max(fx_exp(tv[q].v[0]), fx_exp(tv[q].v[1])));
+      E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
+      Fx x{0ull, 0ll, E < 0x7ff ? E : kFxNaN};
+      if (E < 0x7ff) {
+        // a rotating register file keeps the loop rolled (code size)
+#pragma unroll 1
+        for (int q = 0; q < B && t0 + 32 * q < nt; ++q) {
+          fx_add(x, tv[0].v[0], E);
+          fx_add(x, tv[0].v[1], E);
+#pragma unroll
+          for (int u = 0; u + 1 < B; ++u) tv[u] = tv[u + 1];
         }
-        double t[B];
-#pragma unroll
-        for (int q = 0; q < B; ++q) t[q] = tv[q].hi + tv[q].lo;
-#pragma unroll
-        for (int h = 1; h < B; h <<= 1)
-#pragma unroll
-          for (int q = 0; q + h < B; q += 2 * h) t[q] = t[q] + t[q + h];
-        acc1 = acc1 + t[0];
+        x = fx_warp_sum(x);
       }
-      acc1 = warp_sum(acc1);
-      if (lane == 0) red[v] = acc1;
+      if (nt <= 32 * B) {
+        sum = x;
+      } else {
+        // room for the carries of up to 4096 batches (2^20 tiles): 12 bits
+        if (x.e < kFxNaN) {
+          x.lo = (x.lo >> 12) | ((unsigned long long)x.hi << 52);
+          x.hi >>= 12;
+          x.e += 12;
+        }
+        const int e = max(x.e, sum.e);
+        fx_down(x, e);
+        fx_down(sum, e);
+        sum.lo += x.lo;
+        sum.hi += x.hi + (sum.lo < x.lo ? 1ll : 0ll);
+      }
     }
+    const DD d = fx_dd(sum);
+    if (lane == 0) red[v] = d.hi + d.lo;
   }
 }
 
@@ -257,7 +245,10 @@ __device__ __forceinline__ void precompute_divisions(const SolveState& S, const 
       //   <r', L(p')>    = <r', L(e)> = h,
       //   <L(p'), L(p')> = <L(e), L(e)> + sum_l alpha_l <L(e), L(p^l)> = q + sum_l alpha_l d_l.
       const double ad = lane < kMaxK && lane <= S.nu ? q * red[1 + lane] : 0.0;
-      const double sum = warp_sum(ad);
+      double sum = ad;  // over lanes 0 .. nu
+#pragma unroll 1
+      for (int o = S.nu < 4 ? 2 : 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      sum = __shfl_sync(0xffffffffu, sum, 0);
       const double h = red[2 + S.nu], qq = red[3 + S.nu];
       const double den = qq + sum;
       // use the identities only while they keep three digits of <L(p'),L(p')>
@@ -291,7 +282,7 @@ __device__ int new_slot(const SolveDev<T>& sd, const SolveState& N, int nu) {
 // norm, k dots and, on the mixed path, h and q; INIT: 4).
 template <typename T>
 __device__ __forceinline__ int part_values(const SolveDev<T>& sd) {
-  const int n = sd.mixed ? sd.k + 3 : sd.k + 1;
+  const int n = sd.mixed || sd.band ? sd.k + 3 : sd.k + 1;
   return n > 4 ? n : 4;
 }
 
@@ -310,10 +301,12 @@ __device__ __forceinline__ int part_count(int kind, int nu) {
 }
 
 // The per-solve state machine: consumes the reduced partial sums of the phase
-// that ran last round (S.pending) and decides this round's phase.  Thread 0.
+// that ran last round (S.pending) and decides this round's phase.  One thread.
+// expect: assume the usual outcome of a step round (accepted, the direction's
+// dots from the identities) before its sums are known; see expect_next.
 template <typename T>
 __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState& S, const double* red, const double* qd,
-                                       SolveState& N, Ctx<T>& c) {
+                                       SolveState& N, Ctx<T>& c, bool expect = false) {
   // On entry N is a copy of S and c is zeroed (every pointer a phase may
   // test starts out null); the caller makes both copies block-wide.
   c.kind = K_NONE;
@@ -484,7 +477,7 @@ __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState&
       const double nrm2 = red[0];
       N.nrm2_last = nrm2;
       const double thr2 = sd.mixed ? S.thr2_in : S.thr2;
-      if (nrm2 <= thr2) {  // exit test first (Algorithm 1)
+      if (!expect && nrm2 <= thr2) {  // exit test first (Algorithm 1)
         if (!sd.mixed) {
           N.status = ST_CONVERGED;
           finbuf = S.phiW;
@@ -493,7 +486,7 @@ __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState&
           dbuf = S.phiW;
           to_out = true;
         }
-      } else if (sd.protect && !(nrm2 < S.nrm2_prev)) {  // fault test (Algorithm 1, red part)
+      } else if (!expect && sd.protect && !(nrm2 < S.nrm2_prev)) {  // fault test (Algorithm 1, red part)
         N.fdet = S.fdet + 1;
         N.restarts = S.restarts + 1;
         if (S.ndetect < kMaxDetect) {
@@ -565,9 +558,12 @@ __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState&
           }
           c.pnew = sd.p[ns];
           c.lpnew = sd.Lp[ns];
-          if (sd.mixed && qd[kMaxK + 2] > 0.0) {
-            // mixed path: form p' and take step t + 1 with it in one round
-            // (PF), beta and <L(p'), L(p')> from the identities
+          if ((sd.mixed || (sd.band && !state_flip_near(sd, t))) && (expect || qd[kMaxK + 2] > 0.0)) {
+            // mixed path, and banded FP64 solves away from planned flips (a
+            // flip leaves the cycle's L(p^l) and r' no longer orthogonal, and
+            // beta is formed from the flipped vectors): form p' and take step
+            // t + 1 with it in one round (PF), beta and <L(p'), L(p')> from
+            // the identities
             c.kind = K_PF;
             c.nuo = S.nu;
             N.beta = qd[kMaxK + 1];
@@ -622,7 +618,7 @@ __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState&
       c.eR = sd.e[S.ecur];
       c.LeR = sd.Le[S.ecur];
     }
-    N.ecur = sd.mixed ? (S.ecur ^ 1) : 0;
+    N.ecur = sd.mixed || sd.band ? (S.ecur ^ 1) : 0;
     c.eW = sd.e[N.ecur];
     c.LeW = sd.Le[N.ecur];
   } else if (c.kind == K_PB) {
@@ -659,11 +655,10 @@ __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState&
 
 // The per-direction entries of the context the transition chose (alpha and
 // the p / L(p) slot pointers), one direction per thread: threads 0..kMaxK-1
-// of the block, after the transition.
+// of the block (l), after the transition.
 template <typename T>
 __device__ __forceinline__ void fill_directions(const SolveDev<T>& sd, const SolveState& S, const SolveState& N,
-                                                const double* qd, Ctx<T>& c) {
-  const int l = threadIdx.x;
+                                                const double* qd, Ctx<T>& c, int l) {
   if (l >= kMaxK) return;
   if (c.kind == K_PA || c.kind == K_PF) {
     if (l <= N.nu) c.lp[l] = sd.Lp[N.slot[l]];
@@ -677,6 +672,43 @@ __device__ __forceinline__ void fill_directions(const SolveDev<T>& sd, const Sol
     c.lp[l] = sd.Lp[S.slot[l]];
     c.alpha[l] = (T)qd[l];
   }
+}
+
+// The usual next transition, taken while the grid barrier is waited for: a
+// step round is accepted and followed by PB (FP64 path) or PF (mixed path), PB
+// and RESTORE by PA.  Their buffers, counters and pointers follow from the
+// state alone; only norms, beta and alpha come from the sums.  Whether the
+// sums bear the expectation out is tested by expectation_holds, which also
+// fills them in; if not, the full transition runs as ever.  Takes the serial
+// transition (1.5 us) off the round's critical path.
+__device__ __forceinline__ bool can_expect(const SolveState& S) {
+  return S.active && (S.pending == K_PA || S.pending == K_PF || S.pending == K_PB || S.pending == K_RESTORE);
+}
+// Warp 0, qd from precompute_divisions (in q, lane by lane).
+template <typename T>
+__device__ __forceinline__ bool expectation_holds(const SolveDev<T>& sd, const SolveState& S, const double* red,
+                                                  const double* qd, SolveState& N, Ctx<T>& c) {
+  const int lane = threadIdx.x;
+  if (S.pending == K_PA || S.pending == K_PF) {
+    const double nrm2 = red[0];
+    const double thr2 = sd.mixed ? S.thr2_in : S.thr2;
+    if (nrm2 <= thr2 || (sd.protect && !(nrm2 < S.nrm2_prev)) || (c.kind == K_PF && !(qd[kMaxK + 2] > 0.0))) return false;
+    if (lane == 0) {
+      N.nrm2_last = nrm2;
+      N.nrm2_prev = nrm2;
+      if (c.kind == K_PF) {
+        N.beta = qd[kMaxK + 1];
+        N.lpn2[N.nu] = qd[kMaxK + 2];
+        c.beta = (T)qd[kMaxK + 1];
+      }
+    }
+    if (lane <= S.nu && lane < kMaxK && (c.kind == K_PF || c.kind == K_PB)) c.alpha[lane] = (T)qd[lane];
+  } else if (lane == 0) {  // PB, RESTORE
+    N.beta = qd[kMaxK];
+    N.lpn2[S.nu] = red[1];
+    c.beta = (T)qd[kMaxK];
+  }
+  return true;
 }
 
 // ------------------------------------------------------------ phases
@@ -1342,9 +1374,9 @@ __device__ __forceinline__ void step_stencil(const SolveDev<T>& sd, const Ctx<T>
   if constexpr (kMixed) {
     cta_red_put(ps.cr, 2 + c.nu, ah);
     cta_red_put(ps.cr, 3 + c.nu, aq);
-    cta_red_finish<T>(ps.cr, 4 + c.nu, part_out, write_e ? 0 : 1);
+    cta_red_finish(ps.cr, 4 + c.nu, part_out, write_e ? 0 : 1);
   } else {
-    cta_red_finish<T>(ps.cr, 2 + c.nu, part_out, write_e ? 0 : 1);
+    cta_red_finish(ps.cr, 2 + c.nu, part_out, write_e ? 0 : 1);
   }
 }
 
@@ -1407,7 +1439,7 @@ __device__ __noinline__ void phase_pa_any(const SolveDev<T>& sd, const Ctx<T>& c
     if (mode == 1) {
       store_rows(c.eW, rt.h0, rt.h1, nlon, sm, stride);
       cta_red_put(ps.cr, 0, an);
-      cta_red_finish<T>(ps.cr, 1, part_out);
+      cta_red_finish(ps.cr, 1, part_out);
       return;
     }
   }
@@ -1508,7 +1540,7 @@ __device__ __noinline__ void phase_pb(const SolveDev<T>& sd, const Ctx<T>& c, in
   }
   cta_red_put(ps.cr, 0, a0);
   cta_red_put(ps.cr, 1, a1);
-  cta_red_finish<T>(ps.cr, 2, part_out);
+  cta_red_finish(ps.cr, 2, part_out);
 }
 
 // RESTORE: [phi, r, p, L(p)]^0 <- [phi, r, p, L(p)]^* by copy (the backup
@@ -1547,7 +1579,7 @@ __device__ __noinline__ void phase_restore(const SolveDev<T>& sd, const Ctx<T>& 
   }
   cta_red_put(ps.cr, 0, a0);
   cta_red_put(ps.cr, 1, a1);
-  cta_red_finish<T>(ps.cr, 2, part_out);
+  cta_red_finish(ps.cr, 2, part_out);
 }
 
 // The parts of INIT, inlined into the one-pass phase and the two passes of a
@@ -1729,7 +1761,7 @@ __device__ __forceinline__ void init_partials(PhaseSmem& ps, double* part_out, c
   }
   cta_red_put(ps.cr, 2, a0);
   cta_red_put(ps.cr, 3, a1);
-  cta_red_finish<T>(ps.cr, 4, part_out, full ? 0 : 2);
+  cta_red_finish(ps.cr, 4, part_out, full ? 0 : 2);
 }
 
 // INIT: r0 = L(phi0) - R (FP64 path, phi0 = x0) or r0 = -R_in (mixed inner
@@ -1835,7 +1867,7 @@ __device__ __noinline__ void phase_init_any(const SolveDev<T>& sd, const Ctx<T>&
       cta_red_put(ps.cr, 1, aR64);
     else
       cta_red_put(ps.cr, 1, aR);
-    cta_red_finish<T>(ps.cr, 2, part_out);
+    cta_red_finish(ps.cr, 2, part_out);
     return;
   }
   init_partials<T>(ps, part_out, &an, &aR, a0, a1, mode == 0, c.rin_R && sizeof(T) == 4 ? &aR64 : nullptr);
@@ -1927,7 +1959,7 @@ __device__ __noinline__ void phase_out(const SolveDev<T>& sd, const Ctx<T>& c, i
   }
   cta_red_put(ps.cr, 0, so);
   cta_red_put(ps.cr, 1, sR);
-  cta_red_finish<T>(ps.cr, 2, part_out);
+  cta_red_finish(ps.cr, 2, part_out);
 }
 
 // FIN: write the solution to the caller's x and (FP64 path) the true
@@ -1989,12 +2021,14 @@ __device__ __noinline__ void phase_fin(const SolveDev<T>& sd, const Ctx<T>& c, i
   if constexpr (sizeof(T) == 8)
     cta_red_put(ps.cr, 0, acc);
   else
-    cta_red_put(ps.cr, 0, DD{0.0, 0.0});  // mixed path: no residual formed here
-  cta_red_finish<T>(ps.cr, 1, part_out);
+    cta_red_zero(ps.cr, 0);  // mixed path: no residual formed here
+  cta_red_finish(ps.cr, 1, part_out);
 }
 
 }  // namespace ftgcr
+#if FTGCR_THREADS == 256
 #include "ftgcr_stream.cuh"
+#endif
 namespace ftgcr {
 
 // ------------------------------------------------------------ the kernel
@@ -2032,6 +2066,7 @@ struct KernelSmem {
   double qd[32];
   int prefix[kMaxBatch + 1];
   int bail;
+  int expected;  // N and c hold the expected next transition of S
 };
 
 // Loop state of a CTA (the same in every thread).
@@ -2042,6 +2077,8 @@ struct LoopState {
   int cur = -1;               // solve whose context ks.c holds this round
   int spec_s = -1;            // solve whose partial sums ks.red holds already (speculative)
   bool red_ready = false;
+  bool expected = false;      // ks.S, ks.N, ks.c hold the expected transition of solve last_s
+  int entered = 0;            // solves entered this round
 };
 
 // Entering solve s in a round: its descriptor, its state record and every
@@ -2057,23 +2094,42 @@ __device__ __forceinline__ void enter_solve(SolveDev<T>* const* solves, KernelSm
     __syncthreads();
     ls.cur_sd = s;
   }
-  if (s == ls.last_s && round == ls.last_round + 1)
-    cta_store(&ks.S, &ks.N);
-  else
-    cta_load_cg(&ks.S, ks.sd.st + par);
-  if (!(ls.red_ready && s == ls.spec_s))
-    reduce_partials<T>(ks.sd.part + (long long)(par ^ 1) * ks.sd.nt * kPartStride, ks.sd.nt, part_values(ks.sd),
+  const bool expected = ls.expected && s == ls.last_s && round == ls.last_round + 1;
+  ls.expected = false;
+  ++ls.entered;
+  if (!expected) {
+    if (s == ls.last_s && round == ls.last_round + 1)
+      cta_store(&ks.S, &ks.N);
+    else
+      cta_load_cg(&ks.S, ks.sd.st + par);
+  }
+  if (!(ls.red_ready && s == ls.spec_s)) {
+    reduce_partials(ks.sd.part + (long long)(par ^ 1) * ks.sd.nt * kPartStride, ks.sd.nt, part_values(ks.sd),
                        ks.red);
+    __syncthreads();
+  } else if (!expected) {
+    __syncthreads();
+  }
   ls.red_ready = false;
-  __syncthreads();
-  precompute_divisions(ks.S, ks.red, ks.qd, ks.sd.mixed);
-  cta_store(&ks.N, &ks.S);
-  cta_zero(&ks.c);
-  __syncthreads();
-  if (threadIdx.x == 0) transition(ks.sd, ks.S, ks.red, ks.qd, ks.N, ks.c);
-  __syncthreads();
-  fill_directions(ks.sd, ks.S, ks.N, ks.qd, ks.c);
-  __syncthreads();
+  precompute_divisions(ks.S, ks.red, ks.qd, ks.sd.mixed || ks.sd.band);
+  if (expected) {
+    if (threadIdx.x < 32) {
+      __syncwarp();
+      const bool holds = expectation_holds(ks.sd, ks.S, ks.red, ks.qd, ks.N, ks.c);
+      if (threadIdx.x == 0) ks.expected = holds;
+    }
+    __syncthreads();
+  }
+  if (!expected || !ks.expected) {
+    if (expected) __syncthreads();  // every thread has seen ks.expected, before N and c are rebuilt
+    cta_store(&ks.N, &ks.S);
+    cta_zero(&ks.c);
+    __syncthreads();
+    if (threadIdx.x == 0) transition(ks.sd, ks.S, ks.red, ks.qd, ks.N, ks.c);
+    __syncthreads();
+    fill_directions(ks.sd, ks.S, ks.N, ks.qd, ks.c, threadIdx.x);
+    __syncthreads();
+  }
   ls.cur = s;
   ls.last_s = s;
   ls.last_round = round;
@@ -2089,6 +2145,7 @@ __device__ __forceinline__ void run_phase(KernelSmem<T>& ks, int pass, int s, in
   if constexpr (WIDE != 0 && sizeof(T) == 4) {
     const int mode = ks.sd.split ? 1 + pass : 0;
     if (pass == 1 && mode == 0) return;
+#if FTGCR_THREADS == 256
     if constexpr (WIDE == 2) {
       // streamed solves: the step rounds stream rows; the other rounds run as
       // split rounds over sub-bands
@@ -2101,6 +2158,7 @@ __device__ __forceinline__ void run_phase(KernelSmem<T>& ks, int pass, int s, in
         return;
       }
     }
+#endif
     switch (kind) {
       case K_INIT: phase_init_any<T>(ks.sd, ks.c, s, tau, sm, ks.ps, part_out, mode); return;
       case K_PA: phase_pa_any<T, KB, false>(ks.sd, ks.c, s, tau, sm, ks.ps, part_out, mode); return;
@@ -2143,12 +2201,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_persistent(BatchArgs<T> a
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ KernelSmem<T> ks;
   T* sm = reinterpret_cast<T*>(dsm);
+#if FTGCR_THREADS == 256
   if constexpr (WIDE == 2 && sizeof(T) == 4) stream_init();
+#endif
   const long long round0 = a.ctl->round0;
   const unsigned long long t_start = globaltimer();
   unsigned int nbar = 0;
   LoopState ls;
-  if (threadIdx.x == 0) ks.ps.cs_solve = -1;
+  if (threadIdx.x == 0) {
+    ks.ps.cs_solve = -1;
+    ks.ps.cr.stride = 2;
+  }
   int it = 0;
   for (; it < a.max_rounds; ++it) {
     // watchdog: a kernel that runs far longer than any solve raises the error
@@ -2167,8 +2230,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_persistent(BatchArgs<T> a
     ls.spec_s = spec_s;
     ls.red_ready = spec_s >= 0;
     ls.cur = -1;
+    ls.entered = 0;
     if (spec_s >= 0)
-      reduce_partials<T>(ks.sd.part + (long long)(par ^ 1) * ks.sd.nt * kPartStride, ks.sd.nt, part_values(ks.sd),
+      reduce_partials(ks.sd.part + (long long)(par ^ 1) * ks.sd.nt * kPartStride, ks.sd.nt, part_values(ks.sd),
                          ks.red, 1);
     // tile prefix over active solves (identical in every CTA): warp 0 scans
     // 32 solves at a time
@@ -2233,21 +2297,38 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_persistent(BatchArgs<T> a
             a.diag[blockIdx.x * 4 + 3] = tr_items;
           }
         }
-        run_phase<T, KB, WIDE>(ks, pass, s, tau, sm, ks.sd.part + ((long long)par * ks.sd.nt + tau) * kPartStride,
-                               &a.ctl->err);
-        __syncthreads();
         if (pass == 0 && tau == 0) {
+          // the record for the next round (read after the barrier), stored
+          // before the phase so that its stores overlap the phase's work
           cta_store(ks.sd.st + (par ^ 1), &ks.N);
           if (!ks.N.active) cta_store(ks.sd.result, &ks.N);
           if (threadIdx.x == 0) a.active[(par ^ 1) * a.n + s] = ks.N.active;
-          __syncthreads();
         }
+        run_phase<T, KB, WIDE>(ks, pass, s, tau, sm, ks.sd.part + ((long long)par * ks.sd.nt + tau) * kPartStride,
+                               &a.ctl->err);
+        __syncthreads();
       }
     }
     if (a.trace && threadIdx.x == 0) tr2 = globaltimer();
     if (threadIdx.x == 0 && a.diag) a.diag[blockIdx.x * 4 + 2] = 2;
     ++nbar;
-    const bool ok = grid_barrier(&a.ctl->counter, nbar * gridDim.x, &a.ctl->err, &ks.bail);
+    // a CTA that works on one solve forms its usual next transition meanwhile
+    ls.expected = ls.entered == 1 && can_expect(ks.N);
+    const bool expecting = ls.expected;
+    const bool ok = grid_barrier(&a.ctl->counter, nbar * gridDim.x, &a.ctl->err, &ks.bail, [&] {
+      if (!expecting) return;
+      const int t = threadIdx.x - 32;
+      constexpr int n = kThreads - 32;
+      for (int i = t; i < (int)(sizeof(SolveState) / 8); i += n)
+        reinterpret_cast<long long*>(&ks.S)[i] = reinterpret_cast<const long long*>(&ks.N)[i];
+      for (int i = t; i < (int)(sizeof(Ctx<T>) / 8); i += n) reinterpret_cast<long long*>(&ks.c)[i] = 0;
+      asm volatile("bar.sync 15, %0;" ::"n"(kThreads - 32) : "memory");
+      if (t < 32) {
+        if (t == 0) transition(ks.sd, ks.S, ks.red, ks.qd, ks.N, ks.c, true);
+        __syncwarp();
+        fill_directions(ks.sd, ks.S, ks.N, ks.qd, ks.c, t);
+      }
+    });
     if (a.trace && threadIdx.x == 0 && it < a.trace_rounds) {
       TraceEnt e;
       e.t0 = tr0;

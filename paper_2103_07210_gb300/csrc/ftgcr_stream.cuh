@@ -522,23 +522,6 @@ __device__ __forceinline__ void apply_losses_piece(const SolveDev<float>& sd, lo
   }
 }
 
-// Adds the CTA's sums of values [v0, nv) to the tile's partial sums already
-// in `out` (FP32 path: one double per value).
-__device__ __forceinline__ void cta_red_finish_add(CtaRed& cr, int nv, double* out, int v0) {
-  __syncthreads();
-  if (threadIdx.x >= v0 && threadIdx.x < nv) {
-    const int v = threadIdx.x;
-    double t[kWarps];
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) t[w] = cr.w[w][v].hi + cr.w[w][v].lo;
-#pragma unroll
-    for (int h = 1; h < kWarps; h <<= 1)
-#pragma unroll
-      for (int w = 0; w + h < kWarps; w += 2 * h) t[w] = t[w] + t[w + h];
-    out[2 * v] = out[2 * v] + t[0];
-  }
-}
-
 // The step round (PA, or PF with FUSED) of band tau of a streamed solve.
 // pass 0: every row's axpy, line solve and e, and the stencils of the rows
 // whose neighbours are all in the band; partial sums 0 (||r'||^2) and the
@@ -744,14 +727,14 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
       if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l]);
     cta_red_put(ps.cr, 2 + c.nu, ah);
     cta_red_put(ps.cr, 3 + c.nu, aq);
-    cta_red_finish<float>(ps.cr, 4 + c.nu, part_out);
+    cta_red_finish(ps.cr, 4 + c.nu, part_out);
   } else {
 #pragma unroll
     for (int l = 0; l < KB; ++l)
       if (l <= c.nu) cta_red_put(ps.cr, 1 + l, ad[l]);
     cta_red_put(ps.cr, 2 + c.nu, ah);
     cta_red_put(ps.cr, 3 + c.nu, aq);
-    cta_red_finish_add(ps.cr, 4 + c.nu, part_out, 1);
+    cta_red_finish(ps.cr, 4 + c.nu, part_out, 1, true);
   }
   if (threadIdx.x == 0) g_ss.cph = cph;
 }

@@ -624,6 +624,26 @@ __device__ __forceinline__ T stencil_op(int oracle_order, T v, T ve, T vw, T vn,
   return stencil5<T>(v, ve, vw, vn, vs, txc, txw, tyc, tys, muA, hasN, hasS);
 }
 
+// Exact conversions on the integer pipe (a conversion from or to FP64 takes
+// the FP64 pipe's 18 cycles a warp); what is not a normal number or zero takes
+// the instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 255u;
+  if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+  return (double)f;
+}
+// Round to nearest even; a carry out of the mantissa steps the exponent (up
+// to infinity).
+__device__ __forceinline__ float narrow(double d) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), e = ((h >> 20) & 0x7ffu) - 896u;
+  if (e - 1u < 254u) {
+    const unsigned u = (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29), rem = l & 0x1fffffffu;
+    return __uint_as_float((h & 0x80000000u) | (u + (rem + (u & 1u) > 0x10000000u ? 1u : 0u)));
+  }
+  if ((h << 1 | l) == 0u) return __uint_as_float(h);
+  return (float)d;
+}
 // Shared-memory row layout: element i of a row lives at i + i/32 (one pad
 // word per 32), which keeps both the coalesced sweeps and the per-lane
 // contiguous chunks of the line solve free of bank conflicts.

@@ -1873,90 +1873,222 @@ __device__ __noinline__ void phase_init_any(const SolveDev<T>& sd, const Ctx<T>&
   init_partials<T>(ps, part_out, &an, &aR, a0, a1, mode == 0, c.rin_R && sizeof(T) == 4 ? &aR64 : nullptr);
 }
 
+// Columns i, i + 1 of a row at p + i; v2: 16-byte accesses, else column by
+// column (the second only where it lies in the row).
+struct D2 {
+  double a, b;
+};
+template <bool NC>
+__device__ __forceinline__ D2 ld_d2(const double* p, bool v2, bool two) {
+  D2 r;
+  if (v2) {
+    const double2 q = NC ? __ldg(reinterpret_cast<const double2*>(p)) : __ldcg(reinterpret_cast<const double2*>(p));
+    r.a = q.x, r.b = q.y;
+  } else {
+    r.a = NC ? __ldg(p) : __ldcg(p);
+    r.b = two ? (NC ? __ldg(p + 1) : __ldcg(p + 1)) : 0.0;
+  }
+  return r;
+}
+
 // OUT (mixed): x' = x + d in FP64, r_out = R - L64(x'), ||r_out||^2 (and
-// ||R||^2 the first time), inner right-hand side R_in = (float) r_out.  The
-// tile is walked in sub-bands of at most sd.sub_h rows (each staged with its
-// halo rows) when it is taller than shared memory holds.
+// ||R||^2 the first time), inner right-hand side R_in = (float) r_out.
+//
+// The FP64 pipe bounds this round (a warp instruction every 18 cycles on each
+// SM), so it is laid out to spend few of its instructions.  x' of sub_h + 2
+// rows lies in a ring of rows in shared memory, each formed once (a sub-band's
+// own halo rows cost 5/3 of that on 4096 columns).  A thread takes two columns
+// down the rows of a sub-band: the difference to the north neighbour is, with
+// its sign turned, the next row's to the south, and likewise between its two
+// columns, 2.5 subtractions a point instead of four; the values are the same.
+// Conversions and the test for zero run on the integer pipe.  10.9 FP64
+// instructions a point against 17 (4096 x 2048: 559 to 293 us a round on
+// average, 2048 x 1024: 87 to 76, 1024 x 512: 33 to 29; 360 x 181 is bound by
+// latency, 15 to 15).  Loading a row's coefficients one row ahead gave 5 % on
+// 4096 columns and cost 2 us a round on 360.
 template <typename T>
 __device__ __noinline__ void phase_out(const SolveDev<T>& sd, const Ctx<T>& c, int tau, double* smd, PhaseSmem& ps,
                           double* part_out) {
-  const int nlon = sd.nlon, nlat = sd.nlat, stride = row_stride(nlon);
-  const RowTile rtile = row_tile(nlat, sd.nt, tau);
+  const int n = sd.nlon, nlat = sd.nlat, stride = row_stride(n), P = (n + 1) >> 1;
+  const RowTile rt = row_tile(nlat, sd.nt, tau);
   if (threadIdx.x == 0) ps.cs_solve = -1;  // its FP64 rows overwrite the staged constants
   AccF64 so, sR;
-  const int sub = sd.sub_h > 0 ? sd.sub_h : rtile.j1 - rtile.j0;
-  for (int a = rtile.j0; a < rtile.j1; a += sub) {
-    RowTile rt;
-    rt.j0 = a;
-    rt.j1 = min(a + sub, rtile.j1);
-    rt.h0 = rt.j0 > 0 ? rt.j0 - 1 : 0;
-    rt.h1 = rt.j1 < nlat ? rt.j1 + 1 : nlat;
-    if (a > rtile.j0) __syncthreads();  // the previous sub-band's rows are read
+  // rows by reciprocal: w + 1/2 lies 1 / 2P or more off a multiple of P, far
+  // above the rounding of w < 2^16 times 1 / P
+  const float rP = 1.f / (float)P;
+  const int sub = sd.sub_h > 0 ? sd.sub_h : rt.j1 - rt.j0, ring = sub + 2;
+  const double *xs = c.xsrc, *R = sd.R, *Tx = sd.Tx64, *Ty = sd.Ty64;
+  double* xd = c.xdst;
+  const float* d = reinterpret_cast<const float*>(c.d);
+  float* Rin = reinterpret_cast<float*>(sd.Rin);
+  auto mis = [](const void* q) { return (unsigned)(size_t)q & 15u; };
+  const bool even = !(n & 1), v2 = even && !(mis(xs) | mis(xd) | mis(Tx) | mis(Ty)), v2R = even && !mis(R);
+  const bool none = !xs && !d;  // x' = 0: a zero-guess solve's first OUT
+  // row j, column i at ring slot (j - lo) % ring, element i + 2; the columns
+  // beyond either end of the row are repeated there
+  const int lo = max(rt.j0 - 1, 0);
+  int staged = lo, head = 0;  // next row to form, and its slot
+  int nz1 = 0, nz2 = 0;
+  bool same = c.first;  // ||R||^2 wanted, and so far the same sum
+#pragma unroll 1
+  for (int a = rt.j0; a < rt.j1; a += sub) {
+    const int b = min(a + sub, rt.j1), top = min(b + 1, nlat);
+    if (a > rt.j0) __syncthreads();  // the rows overwritten are read
     int nz = 0;
     {
-      // x' = x + d over the sub-band and its halo rows, as one flat loop so
-      // that each thread keeps several loads in flight
-      const int nrows = rt.h1 - rt.h0, total = nrows * nlon;
-      constexpr int U = 4;
-      for (int b = threadIdx.x; b < total; b += U * kThreads) {
-        double xv[U];
+      const int total = (top - staged) * P;
+      constexpr int U = kThreads > 256 ? 2 : 4;
+#pragma unroll 1
+      for (int q0 = threadIdx.x; q0 < total; q0 += U * kThreads) {
+        D2 xv[U];
+        int jr[U], ii[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int idx = b + u * kThreads;
-          if (idx < total) {
-            const long long g = (long long)rt.h0 * nlon + idx;
-            xv[u] = c.xsrc ? ldcg(c.xsrc + g) : 0.0;  // x = 0 before a zero-guess solve's first OUT
-            if (c.d) xv[u] = xv[u] + (double)ldcg(c.d + g);
+          const int w = q0 + u * kThreads;
+          jr[u] = __float2int_rz(((float)w + 0.5f) * rP);
+          ii[u] = 2 * (w - jr[u] * P);
+          xv[u].a = xv[u].b = 0.0;
+          if (w < total && xs) xv[u] = ld_d2<false>(xs + ((long long)(staged + jr[u]) * n + ii[u]), v2, ii[u] + 1 < n);
+        }
+        if (d) {
+          float2 dv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            dv[u] = make_float2(0.f, 0.f);
+            if (q0 + u * kThreads < total) {
+              const float* p = d + ((long long)(staged + jr[u]) * n + ii[u]);
+              if (even) dv[u] = __ldcg(reinterpret_cast<const float2*>(p));
+              else {
+                dv[u].x = __ldcg(p);
+                if (ii[u] + 1 < n) dv[u].y = __ldcg(p + 1);
+              }
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            xv[u].a = xv[u].a + widen(dv[u].x);
+            xv[u].b = xv[u].b + widen(dv[u].y);
           }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int idx = b + u * kThreads;
-          if (idx < total) {
-            const int jr = idx / nlon, i = idx - jr * nlon;
-            smd[jr * stride + sk(i)] = xv[u];
-            nz |= xv[u] != 0.0;
-            const int j = rt.h0 + jr;
-            if (j >= rt.j0 && j < rt.j1) c.xdst[(long long)rt.h0 * nlon + idx] = xv[u];
+          if (q0 + u * kThreads >= total) continue;
+          const int j = staged + jr[u], e = ii[u];
+          const bool two = e + 1 < n;
+          if (!none) {
+            int slot = head + jr[u];
+            if (slot >= ring) slot -= ring;
+            double* row = smd + slot * stride + 2;
+            if (e == 0) row[n] = xv[u].a;
+            if (two) *reinterpret_cast<double2*>(row + e) = make_double2(xv[u].a, xv[u].b);
+            else row[e] = xv[u].a;
+            if (e + 2 >= n) row[-1] = two ? xv[u].b : xv[u].a;
+            nz |= ((__double_as_longlong(xv[u].a) | __double_as_longlong(xv[u].b)) << 1) != 0;
+          }
+          if (j >= rt.j0 && j < rt.j1) {
+            double* p = xd + ((long long)j * n + e);
+            if (v2) *reinterpret_cast<double2*>(p) = make_double2(xv[u].a, xv[u].b);
+            else {
+              p[0] = xv[u].a;
+              if (two) p[1] = xv[u].b;
+            }
           }
         }
       }
+      head += top - staged;
+      if (head >= ring) head -= ring;
+      staged = top;
     }
-    // a sub-band whose x' (halo included) is all zero, as at the start of a
-    // solve from a zero guess, has L64(x') = 0: skip the FP64 stencil
-    const bool zero = !__syncthreads_or(nz);
-    for (int j = rt.j0; j < rt.j1; ++j) {
-      const long long base = (long long)j * nlon;
-      const double* row = smd + (j - rt.h0) * stride;
-      const bool hasN = j < nlat - 1, hasS = j > 0;
+    // rows (halo rows included) that are all zero, as at the start of a solve
+    // from a zero guess, have L64(x') = 0: no FP64 stencil
+    nz = __syncthreads_or(nz);
+    const bool zero = !(nz | nz1 | nz2);  // (a row lies in the ring for up to three sub-bands)
+    nz2 = nz1, nz1 = nz;
+    if (same && !zero) {
+      same = false;
+      sR = so;
+    }
+    // strips of rows, so that every thread has some
+    const int rows = b - a, strips = max(1, min(rows, kThreads / P)), sr = (rows + strips - 1) / strips;
+#pragma unroll 1
+    for (int q = threadIdx.x; q < strips * P; q += kThreads) {
+      const int st = __float2int_rz(((float)q + 0.5f) * rP), i = 2 * (q - st * P);
+      const int j0 = a + st * sr, j1 = min(j0 + sr, b);
+      const bool two = i + 1 < n;
       if (zero) {
-        for (int i = threadIdx.x; i < nlon; i += kThreads) {
-          const long long g = base + i;
-          const double Rv = ldcg(sd.R + g);
-          const double ro = Rv - 0.0;
-          sd.Rin[g] = (T)ro;
-          so.add(ro, ro);
-          if (c.first) sR.add(Rv, Rv);
+#pragma unroll 4
+        for (int j = j0; j < j1; ++j) {
+          const long long g = (long long)j * n + i;
+          const D2 r = ld_d2<false>(R + g, v2R, two);
+          so.add(r.a, r.a);
+          so.add(r.b, r.b);
+          if (c.first && !same) {
+            sR.add(r.a, r.a);
+            sR.add(r.b, r.b);
+          }
+          if (even) *reinterpret_cast<float2*>(Rin + g) = make_float2(narrow(r.a), narrow(r.b));
+          else {
+            Rin[g] = narrow(r.a);
+            if (two) Rin[g + 1] = narrow(r.b);
+          }
         }
         continue;
       }
-      for (int i = threadIdx.x; i < nlon; i += kThreads) {
-        const long long g = base + i;
-        const int ie = (i + 1 == nlon) ? 0 : i + 1;
-        const int iw = (i == 0) ? nlon - 1 : i - 1;
-        const double v = row[sk(i)];
-        const double Lx = stencil5_fma(v, row[sk(ie)], row[sk(iw)], hasN ? row[stride + sk(i)] : 0.0,
-                                       hasS ? row[-stride + sk(i)] : 0.0, __ldg(sd.Tx64 + g),
-                                       __ldg(sd.Tx64 + base + iw), hasN ? __ldg(sd.Ty64 + g) : 0.0,
-                                       hasS ? __ldg(sd.Ty64 + g - nlon) : 0.0, __ldg(sd.muA64 + j), hasN, hasS);
-        const double Rv = ldcg(sd.R + g);
-        const double ro = Rv - Lx;
-        sd.Rin[g] = (T)ro;
-        so.add(ro, ro);
-        if (c.first) sR.add(Rv, Rv);
+      if (j0 >= j1) continue;
+      int slot = (j0 - lo) % ring;
+      const double* row = smd + slot * stride + 2 + i;
+      D2 v{row[0], row[1]}, s{0.0, 0.0}, tys{0.0, 0.0};  // s: south differences, sign turned
+      if (j0 > 0) {
+        const double* rs = smd + (slot > 0 ? slot - 1 : ring - 1) * stride + 2 + i;
+        s.a = v.a - rs[0], s.b = v.b - rs[1];
+        tys = ld_d2<true>(Ty + ((long long)(j0 - 1) * n + i), v2, two);
+      }
+#pragma unroll 1
+      for (int j = j0; j < j1; ++j) {
+        const long long g = (long long)j * n + i;
+        const D2 tx = ld_d2<true>(Tx + g, v2, two);
+        const double txw = __ldg(Tx + (i == 0 ? g + n - 1 : g - 1));
+        D2 ty{0.0, 0.0};
+        if (j < nlat - 1) ty = ld_d2<true>(Ty + g, v2, two);
+        const D2 r = ld_d2<false>(R + g, v2R, two);
+        const double mu = __ldg(sd.muA64 + j);
+        const double vw = row[-1], ve = row[2];
+        if (++slot == ring) slot = 0;
+        row = smd + slot * stride + 2 + i;
+        const double dm = v.b - v.a;
+        D2 vn{0.0, 0.0}, dn{0.0, 0.0};
+        double La = -mu * v.a, Lb = -mu * v.b;
+        if (j > 0) {
+          La = fma(tys.a, -s.a, La);
+          Lb = fma(tys.b, -s.b, Lb);
+        }
+        if (j < nlat - 1) {
+          vn.a = row[0], vn.b = row[1];
+          dn.a = vn.a - v.a, dn.b = vn.b - v.b;
+          La = fma(ty.a, dn.a, La);
+          Lb = fma(ty.b, dn.b, Lb);
+        }
+        La = fma(txw, vw - v.a, La);
+        Lb = fma(tx.a, -dm, Lb);
+        La = fma(tx.a, dm, La);
+        Lb = fma(tx.b, ve - v.b, Lb);
+        const double ra = r.a - La, rb = r.b - Lb;
+        so.add(ra, ra);
+        if (two) so.add(rb, rb);
+        if (c.first) {
+          sR.add(r.a, r.a);
+          sR.add(r.b, r.b);
+        }
+        if (even) *reinterpret_cast<float2*>(Rin + g) = make_float2(narrow(ra), narrow(rb));
+        else {
+          Rin[g] = narrow(ra);
+          if (two) Rin[g + 1] = narrow(rb);
+        }
+        s = dn, v = vn, tys = ty;
       }
     }
   }
+  if (same) sR = so;
   cta_red_put(ps.cr, 0, so);
   cta_red_put(ps.cr, 1, sR);
   cta_red_finish(ps.cr, 2, part_out);

@@ -2279,14 +2279,30 @@ __device__ __forceinline__ void run_phase(KernelSmem<T>& ks, int pass, int s, in
     if (pass == 1 && mode == 0) return;
 #if FTGCR_THREADS == 256
     if constexpr (WIDE == 2) {
-      // streamed solves: the step rounds stream rows; the other rounds run as
+      // streamed solves: the step rounds stream rows, and so does INIT unless
+      // flips of the first step fall into the band; the other rounds run as
       // split rounds over sub-bands
+      if (ks.sd.split == 2 && kind == K_INIT && (ks.c.zero_guess || ks.c.rin_R)) {
+        bool clean = true;
+        if (ks.sd.nfaults) {
+          if (threadIdx.x == 0)
+            ks.ps.nfl = collect_flips(ks.sd, ks.c.t, kStateVecs, (long long)row_start(ks.sd.nlat, ks.sd.nt, tau) * ks.sd.nlon,
+                                      (long long)row_start(ks.sd.nlat, ks.sd.nt, tau + 1) * ks.sd.nlon, ks.ps.fl);
+          __syncthreads();
+          clean = ks.ps.nfl == 0;
+          __syncthreads();
+        }
+        if (clean) {
+          phase_stream<1, K_INIT>(ks.sd, ks.c, tau, sm, ks.ps, part_out, pass, err);
+          return;
+        }
+      }
       if (ks.sd.split == 2 && kind == K_PA) {
-        phase_stream<KB, false>(ks.sd, ks.c, tau, sm, ks.ps, part_out, pass, err);
+        phase_stream<KB, K_PA>(ks.sd, ks.c, tau, sm, ks.ps, part_out, pass, err);
         return;
       }
       if (ks.sd.split == 2 && kind == K_PF) {
-        phase_stream<KB, true>(ks.sd, ks.c, tau, sm, ks.ps, part_out, pass, err);
+        phase_stream<KB, K_PF>(ks.sd, ks.c, tau, sm, ks.ps, part_out, pass, err);
         return;
       }
     }

@@ -309,9 +309,11 @@ __device__ __forceinline__ void cp_async_wait_n(int n) {
 }
 
 // Operand row v of an axpy stage.
-template <bool FUSED>
-__device__ __forceinline__ const float* ax_src(const Ctx<float>& c, int v) {
-  if constexpr (FUSED) {
+template <int KIND>
+__device__ __forceinline__ const float* ax_src(const SolveDev<float>& sd, const Ctx<float>& c, int v) {
+  if constexpr (KIND == K_INIT) {
+    return sd.Rin;
+  } else if constexpr (KIND == K_PF) {
     if (v == 0) return c.LeR;
     if (v == 1) return c.rC;
     if (v == 2) return c.eR;
@@ -329,10 +331,29 @@ __device__ __forceinline__ const float* ax_src(const Ctx<float>& c, int v) {
 // stage buffer `buf` (shared address), and, for a stencil stage, lane 0's
 // copy of the Tx element west of its warp's columns into `lead`.  The
 // operand rows come from the pass's tables (tab: axpy or stencil).
+// R64 (INIT from the caller's R): the axpy stage's operand rows 0 and 1 hold
+// the four columns in FP64 (columns 0, 1 and 2, 3; 8-byte copies where R is
+// not 16-byte aligned).
 __device__ __forceinline__ void stream_copy(const float* const* tab, const float* Tx, int n, int nlat, int type,
-                                            int row, int ch, int sub, int nv, unsigned buf, unsigned lead) {
+                                            int row, int ch, int sub, int nv, unsigned buf, unsigned lead,
+                                            const double* R64) {
   const int c0 = ch * kCW, i4 = 4 * (int)threadIdx.x;
   const long long ro = (long long)row * n;
+  if (R64 && type == 0) {
+    if (c0 + i4 >= n) return;
+    const double* p = R64 + ro + c0 + i4;
+    const unsigned d0 = buf + 4u * (unsigned)i4, d1 = d0 + 4u * (unsigned)kCW;
+    if (((size_t)R64 & 15u) == 0) {
+      cp_async16_nc(d0, p);
+      cp_async16_nc(d1, p + 2);
+    } else {
+#pragma unroll
+      for (int w = 0; w < 4; ++w)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((w < 2 ? d0 : d1) + 8u * (unsigned)(w & 1)), "l"(p + w)
+                     : "memory");
+    }
+    return;
+  }
   const int v0 = sub * kNVS;
   if (type == 1 && sub == 0 && (threadIdx.x & 31) == 0) {
     const int w0 = c0 + 128 * (int)(threadIdx.x >> 5);
@@ -358,20 +379,46 @@ struct AxRegs {
 // the PA / PF axpy of the other round layouts).  After the last sub-stage:
 // the flips of the step, r'' and phi'', the norm, the state vectors of the
 // row written, r'' into the row buffer.
-template <bool FUSED>
+template <int KIND>
 __device__ __forceinline__ void stream_ax(int n, int lcb, int P, const PhaseSmem& ps, unsigned buf, int row, int ch,
-                                          int sub, int nv, unsigned rb, AxRegs& x, Acc<float>& an) {
+                                          int sub, int nv, unsigned rb, AxRegs& x, Acc<float>& an, bool r64,
+                                          AccF64& aR) {
   const int c0 = ch * kCW, i4 = 4 * (int)threadIdx.x;
   if (c0 + i4 >= n) return;
   const int v0 = sub * kNVS;
   auto S = [&](int q) { return lds4(buf + 4u * (unsigned)(q * kCW + i4)); };
+  if constexpr (KIND == K_INIT) {  // r0 = -R_in, phi = 0
+    const long long g = (long long)row * n + c0 + i4;
+    V16<float> rn = S(0), z;
+    if (r64) {  // r0 = -(float)R, and ||R||^2
+      const V16<float> hi = S(1);
+      double R[4];
+      memcpy(R, &rn, 16);
+      memcpy(R + 2, &hi, 16);
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        rn.v[w] = narrow(R[w]);
+        aR.add(R[w], R[w]);
+      }
+    }
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      rn.v[w] = -rn.v[w];
+      z.v[w] = 0.f;
+      an.add(rn.v[w], rn.v[w]);
+    }
+    stv(g_ss.out[2] + g, rn);
+    stv(g_ss.out[3] + g, z);
+    sts4(rb + 4u * (unsigned)pk(c0 + i4, lcb, P), rn);
+    return;
+  }
   if (sub == 0) {
     x.ln = S(0);
     x.rr = S(1);
     x.pn = S(2);
     x.ph = S(3);
   }
-  if constexpr (FUSED) {
+  if constexpr (KIND == K_PF) {
 #pragma unroll
     for (int q = 0; q < kNVS; q += 2) {
       const int v = v0 + q;
@@ -391,7 +438,7 @@ __device__ __forceinline__ void stream_ax(int n, int lcb, int P, const PhaseSmem
   const float beta = g_ss.beta;
   const int nfl = ps.nfl;
   V16<float> rn, fn;
-  if constexpr (FUSED) {
+  if constexpr (KIND == K_PF) {
     if (nfl) {
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
@@ -409,7 +456,7 @@ __device__ __forceinline__ void stream_ax(int n, int lcb, int P, const PhaseSmem
     fn.v[w] = fmaf(beta, x.pn.v[w], x.ph.v[w]);
     an.add(rn.v[w], rn.v[w]);
   }
-  if constexpr (FUSED) {
+  if constexpr (KIND == K_PF) {
     stv(g_ss.out[0] + g, x.pn);
     stv(g_ss.out[1] + g, x.ln);
   }
@@ -522,7 +569,9 @@ __device__ __forceinline__ void apply_losses_piece(const SolveDev<float>& sd, lo
   }
 }
 
-// The step round (PA, or PF with FUSED) of band tau of a streamed solve.
+// The step round (PA or PF) of band tau of a streamed solve, or its INIT where
+// no flip of the first step falls into the band (4096 x 2048: 252 to 153 us as
+// split rounds, streamed).
 // pass 0: every row's axpy, line solve and e, and the stencils of the rows
 // whose neighbours are all in the band; partial sums 0 (||r'||^2) and the
 // dots of those rows.  pass 1 (after a grid barrier): the stencils of the
@@ -531,15 +580,18 @@ __device__ __forceinline__ void apply_losses_piece(const SolveDev<float>& sd, lo
 // (32 (C + 4) floats each), the constants c, 1/w, z of one row (the same
 // layout), sd.nslot stage buffers of
 // kNVS * kCW floats, then the Tx leads (sd.nslot x 8 x 16 bytes).
-template <int KB, bool FUSED>
+template <int KB, int KIND>
 __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<float>& c, int tau, float* sm,
                                           PhaseSmem& ps, double* part_out, int pass, int* err) {
   const int n = sd.nlon, nlat = sd.nlat, C = sd.C, P = C + 4, lcb = __ffs(C) - 1;
   const int stride = 32 * P;  // a piece-major row
   const int j0 = row_start(nlat, sd.nt, tau), j1 = row_start(nlat, sd.nt, tau + 1);
   const int nch = (n + kCW - 1) / kCW, nbuf = sd.nslot, D = nbuf - 1;
-  const int nv_ax = FUSED ? 4 + 2 * (c.nuo + 1) : 4;
-  const int nv_st = 5 + c.nu;
+  constexpr bool kInit = KIND == K_INIT;
+  const int nv_ax = kInit ? 1 : KIND == K_PF ? 4 + 2 * (c.nuo + 1) : 4;
+  const int nv_st = kInit ? 4 : 5 + c.nu;
+  float* const ebnd = kInit ? sd.e[0] : c.eW;     // e of the band's edge rows, for the neighbours
+  float* const efull = kInit ? c.pnew : c.eW;     // e of every row (INIT: p0)
   const int ns_ax = (nv_ax + kNVS - 1) / kNVS, ns_st = (nv_st + kNVS - 1) / kNVS;
   float* ebuf = sm;
   float* cst = sm + 3 * stride;
@@ -548,7 +600,12 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
   const unsigned ring_s = smem_addr(ring);
   const unsigned lead_s = smem_addr(ring + (size_t)nbuf * kNVS * kCW);
   const unsigned per = 4u * (unsigned)stride;  // bytes of one constants row
-  auto interior = [&](int i) { return (i == 0 || i - 1 >= j0) && (i == nlat - 1 || i + 1 < j1); };
+  // rows whose stencil is formed in pass 0.  The last row of the grid only where
+  // its stencil does not come straight after its axpy, whose r' its stages (in
+  // flight before that axpy ran) would not hold
+  auto interior = [&](int i) {
+    return (i == 0 || i - 1 >= j0) && (i < nlat - 1 ? i + 1 < j1 : i > 0 && (i == 1 || i - 2 >= j0));
+  };
   if (threadIdx.x == 0) {
     ps.cs_solve = -1;  // the dynamic shared memory is laid out for this phase
     int m = 0;
@@ -558,7 +615,7 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
         if (j - 1 >= j0 && interior(j - 1)) g_ss.rl[m++] = ((j - 1) << 1) | 1;
       }
       if (j1 == nlat && j1 - 1 >= j0 && interior(j1 - 1)) g_ss.rl[m++] = ((j1 - 1) << 1) | 1;
-      ps.nfl = collect_flips(sd, c.t, FUSED ? (kStateVecs | (1u << V_E)) : (1u << V_E), (long long)j0 * n,
+      ps.nfl = kInit ? 0 : collect_flips(sd, c.t, KIND == K_PF ? (kStateVecs | (1u << V_E)) : (1u << V_E), (long long)j0 * n,
                              (long long)j1 * n, ps.fl);
     } else {
       if (!interior(j0)) g_ss.rl[m++] = (j0 << 1) | 1;
@@ -568,7 +625,7 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
   }
   if ((int)threadIdx.x < j1 - j0) g_ss.muA[threadIdx.x] = __ldg(sd.muA + j0 + threadIdx.x);
   // the pass's operand tables, outputs and coefficients
-  if ((int)threadIdx.x < nv_ax) g_ss.tab_ax[threadIdx.x] = ax_src<FUSED>(c, threadIdx.x);
+  if ((int)threadIdx.x < nv_ax) g_ss.tab_ax[threadIdx.x] = ax_src<KIND>(sd, c, threadIdx.x);
   if ((int)threadIdx.x >= 64 && (int)threadIdx.x < 64 + nv_st) {
     const int v = threadIdx.x - 64;
     g_ss.tab_st[v] = v == 0 ? sd.Tx : v == 1 ? sd.Ty : v == 2 ? sd.Ty - n : v == 3 ? c.rW : c.lp[v - 4];
@@ -579,7 +636,7 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
     g_ss.out[1] = c.lpnew;
     g_ss.out[2] = c.rW;
     g_ss.out[3] = c.phiW;
-    g_ss.out[4] = c.LeW;
+    g_ss.out[4] = kInit ? c.lpnew : c.LeW;
     g_ss.beta = c.beta;
   }
   __syncthreads();
@@ -604,7 +661,7 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
       const int e = g_ss.rl[pi], type = e & 1, row = e >> 1;
       const int b = pidx % nbuf;
       stream_copy(type ? g_ss.tab_st : g_ss.tab_ax, sd.Tx, n, nlat, type, row, pc, psb, type ? nv_st : nv_ax,
-                  ring_s + 4u * (unsigned)(b * kNVS * kCW), lead_s + 128u * (unsigned)b);
+                  ring_s + 4u * (unsigned)(b * kNVS * kCW), lead_s + 128u * (unsigned)b, kInit && c.rin_R ? sd.R : nullptr);
       if (++psb == (type ? ns_st : ns_ax)) {
         psb = 0;
         if (++pc == nch) {
@@ -618,6 +675,7 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
   };
   for (int d = 0; d < D; ++d) issue_next();
   Acc<float> an, ah, aq;
+  AccF64 aR;
   Acc<float> ad[KB];
   int cidx = 0;
   bool fail = false;
@@ -634,9 +692,12 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
         // the three e rows, the neighbour's included (plain loads; this row's
         // stage copies are in flight meanwhile)
         __syncthreads();  // the previous row's stencil has read them
-        if (row > 0) stage_piece_row(c.eW, row - 1, n, lcb, P, smem_addr(ebuf));
-        stage_piece_row(c.eW, row, n, lcb, P, smem_addr(ebuf + stride));
-        if (row < nlat - 1) stage_piece_row(c.eW, row + 1, n, lcb, P, smem_addr(ebuf + 2 * stride));
+        // (a row whose stencil pass 0 formed was written by it, the others by
+        // their line solve)
+        auto esrc = [&](int q) { return kInit && q >= j0 && q < j1 && interior(q) ? efull : ebnd; };
+        if (row > 0) stage_piece_row(esrc(row - 1), row - 1, n, lcb, P, smem_addr(ebuf));
+        stage_piece_row(ebnd, row, n, lcb, P, smem_addr(ebuf + stride));
+        if (row < nlat - 1) stage_piece_row(esrc(row + 1), row + 1, n, lcb, P, smem_addr(ebuf + 2 * stride));
         __syncthreads();
         eS = smem_addr(ebuf);
         eC = smem_addr(ebuf + stride);
@@ -660,10 +721,10 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
         const int b = cidx % nbuf;
         const unsigned buf = ring_s + 4u * (unsigned)(b * kNVS * kCW);
         if (type == 0)
-          stream_ax<FUSED>(n, lcb, P, ps, buf, row, ch, sb, nv, rb, xa, an);
+          stream_ax<KIND>(n, lcb, P, ps, buf, row, ch, sb, nv, rb, xa, an, kInit && c.rin_R, aR);
         else
           stream_st<KB>(n, nlat, lcb, P, buf, lead_s + 128u * (unsigned)b, row, ch, sb, nv, eC, eN, eS, muA, xs, ad,
-                        ah, aq, pass == 0 ? c.eW : nullptr);
+                        ah, aq, kInit || pass == 0 ? efull : nullptr);
         ++cidx;
       }
     }
@@ -704,12 +765,12 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
         rowbuf[pk(i, lcb, P)] = flip_bits(rowbuf[pk(i, lcb, P)], ps.fl[q].bit);
       }
     }
-    if (sd.nlosses) {
+    if (!kInit && sd.nlosses) {
       __syncthreads();
       apply_losses_piece(sd, c.t, row, rowbuf, lcb, P);
     }
-    if (ps.nfl || sd.nlosses) __syncthreads();  // thread 0's flips before any reader
-    if (!interior(row)) store_piece_row(c.eW, row, n, lcb, P, rb);  // else stored by its stencil
+    if (!kInit && (ps.nfl || sd.nlosses)) __syncthreads();  // thread 0's flips before any reader
+    if (!interior(row)) store_piece_row(ebnd, row, n, lcb, P, rb);  // else stored by its stencil
   }
   cp_async_wait_all();  // the groups still open are empty unless the pass failed
   if (fail) {
@@ -720,7 +781,15 @@ __device__ __noinline__ void phase_stream(const SolveDev<float>& sd, const Ctx<f
     }
     return;
   }
-  if (pass == 0) {
+  if constexpr (kInit) {  // ||r0||^2, ||R||^2 (from R), the first dots
+    if (pass == 0) {
+      cta_red_put(ps.cr, 0, an);
+      cta_red_put(ps.cr, 1, aR);
+    }
+    cta_red_put(ps.cr, 2, ah);
+    cta_red_put(ps.cr, 3, aq);
+    cta_red_finish(ps.cr, 4, part_out, pass ? 2 : 0, pass != 0);
+  } else if (pass == 0) {
     cta_red_put(ps.cr, 0, an);
 #pragma unroll
     for (int l = 0; l < KB; ++l)

@@ -1306,12 +1306,12 @@ struct TeamPlan {
   std::vector<int> order;    // solves (indices into the argument), team by team
   int teams = 0;
 };
-void plan_teams(const std::vector<long long>& points, const std::vector<int>& nt, int sms, TeamPlan* out) {
+void plan_teams(const std::vector<long long>& points, const std::vector<int>& nt, int sms, int most_teams, TeamPlan* out) {
   const int n = (int)points.size();
   std::vector<int> by(n);
   for (int i = 0; i < n; ++i) by[i] = i;
   std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return points[a] > points[b]; });
-  const int teams = std::max(1, std::min(n, sms / kTeamMin));
+  const int teams = std::max(1, std::min({n, sms / kTeamMin, most_teams}));
   // sizes: one CTA each, then one by one to the team with the most points per CTA
   std::vector<int> size(teams, 1);
   for (int left = sms - teams; left > 0; --left) {
@@ -1390,6 +1390,20 @@ int solve_async_impl(ftgcr_handle* h, const double* R, const double* x0, double*
 }
 
 // The schedule of a banded launch, filled like the solve table.
+// The launches of a batch or an epoch: 0 the solves of the other kernels, 1
+// banded solves side by side in teams, 2 banded solves of kWholePoints or more,
+// which take all CTAs one after another: on a few CTAs such a solve reads its
+// vectors from L2 or memory, on all of them its bands stay on chip.  Smaller
+// ones leave CTAs idle or pay for barriers among all.  The line lies between
+// 512 x 256 and 1024 x 512 points: ms with none / 2048 x 1024 / 1024 x 512 and
+// up / 512 x 256 and up taken whole, 32 mixed solves served 37.5 / 23.6 / 21.5 /
+// 23.3, 21 FP64 ones 52.3 / 43.0 / 40.7 / 42.3, a batch of 128 mixed solves (to
+// 1024 x 512) 36.4 / 36.4 / 33.6 / 40.7, of 28 FP64 ones 29.4 / 29.4 / 23.8 / 24.6.
+constexpr long long kWholePoints = 1LL << 18;
+int launch_class(const ftgcr_handle* h) {
+  if (h->wide != kWideBand) return 0;
+  return h->N >= kWholePoints ? 2 : 1;
+}
 constexpr int kMaxTeamCtas = 256;
 struct TeamTable {
   TeamCta cta[kMaxTeamCtas];
@@ -1411,7 +1425,8 @@ __global__ void k_fill_teams(TeamTable t, TeamCta* d_cta) {
 template <typename T>
 int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, double* const* x,
                      const ftgcr_fault_plan* const* plans, int n_all, cudaStream_t st) {
-  for (int band = 0; band < 2; ++band) {
+  for (int cls = 0; cls < 3; ++cls) {
+    const bool band = cls != 0;
     std::vector<int> id;  // this launch's solves
     int kb = 4;
     size_t smem = 1;
@@ -1419,7 +1434,7 @@ int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, doub
     int max_outer = 0, split = 0;
     for (int i = 0; i < n_all; ++i) {
       const ftgcr_handle* h = hs_all[i];
-      if ((h->wide == kWideBand) != (band == 1)) continue;
+      if (launch_class(h) != cls) continue;
       id.push_back(i);
       split = std::max(split, h->wide);
       kb = std::max(kb, kbound(h->k));
@@ -1446,7 +1461,7 @@ int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, doub
         points.push_back(hs_all[i]->N);
         nts.push_back(hs_all[i]->nt);
       }
-      plan_teams(points, nts, std::min(di.sms, kMaxTeamCtas), &tp);
+      plan_teams(points, nts, std::min(di.sms, kMaxTeamCtas), cls == 2 ? 1 : kMaxTeamCtas, &tp);
       grid = (int)tp.cta.size();
     }
     const size_t b_solves = align256(sizeof(void*) * n), b_nt = align256(sizeof(int) * n),
@@ -1571,7 +1586,10 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
   t->h_ctl_out->err = 0;
   t->h_ctl_out->round_end = t->round;
   t->h_bctl->err = 0;
-  for (int band = 0; band < 2; ++band) {
+  int border = 0;          // solves placed in banded launches
+  bool ctl_ready = false;  // their control block is reset
+  for (int cls = 0; cls < 3; ++cls) {
+    const bool band = cls != 0;
     int kb = 4;
     size_t smem = 1;
     long long tiles = 0;
@@ -1579,7 +1597,7 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
     std::vector<int> id;
     for (int s = 0; s < t->n; ++s) {
       const ftgcr_handle* h = t->slot[s];
-      if (!h || (h->wide == kWideBand) != (band == 1)) continue;
+      if (!h || launch_class(h) != cls) continue;
       id.push_back(s);
       split = std::max(split, h->wide);
       kb = std::max(kb, kbound(h->k));
@@ -1601,16 +1619,21 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
         nts.push_back(t->slot[s]->nt);
       }
       TeamPlan tp;
-      plan_teams(points, nts, std::min(device_info(t->dev).sms, kMaxTeamCtas), &tp);
+      plan_teams(points, nts, std::min(device_info(t->dev).sms, kMaxTeamCtas), cls == 2 ? 1 : kMaxTeamCtas, &tp);
       const int grid = (int)tp.cta.size();
-      // the previous launch, whose copies read these, has been collected
-      for (int i = 0; i < grid; ++i) t->h_bcta[i] = tp.cta[i];
-      for (size_t i = 0; i < tp.order.size(); ++i) t->h_border[i] = id[tp.order[i]];
-      CK(cudaMemcpyAsync(t->d_bcta, t->h_bcta, sizeof(TeamCta) * grid, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(t->d_border, t->h_border, sizeof(int) * tp.order.size(), cudaMemcpyHostToDevice, st));
+      // the previous epoch, whose copies read these, has been collected; each
+      // class has its own part
+      TeamCta *h_cta = t->h_bcta + (cls - 1) * kMaxTeamCtas, *d_cta = t->d_bcta + (cls - 1) * kMaxTeamCtas;
+      int *h_ord = t->h_border + border, *d_ord = t->d_border + border;
+      border += (int)tp.order.size();
+      for (int i = 0; i < grid; ++i) h_cta[i] = tp.cta[i];
+      for (size_t i = 0; i < tp.order.size(); ++i) h_ord[i] = id[tp.order[i]];
+      CK(cudaMemcpyAsync(d_cta, h_cta, sizeof(TeamCta) * grid, cudaMemcpyHostToDevice, st));
+      CK(cudaMemcpyAsync(d_ord, h_ord, sizeof(int) * tp.order.size(), cudaMemcpyHostToDevice, st));
       CK(cudaMemsetAsync(t->d_bcnt, 0, 128 * (size_t)tp.teams, st));
-      CK(cudaMemsetAsync(t->d_bctl, 0, sizeof(LaunchCtl), st));
-      rc = launch_band<T>(kb, (SolveDev<T>* const*)t->d_solves, t->d_bact, t->d_bcta, t->d_border, t->d_bcnt, t->d_bctl,
+      if (!ctl_ready) CK(cudaMemsetAsync(t->d_bctl, 0, sizeof(LaunchCtl), st));
+      ctl_ready = true;
+      rc = launch_band<T>(kb, (SolveDev<T>* const*)t->d_solves, t->d_bact, d_cta, d_ord, t->d_bcnt, t->d_bctl,
                           t->d_diag, max_rounds, grid, smem, st);
       if (rc) return rc;
       CK(cudaMemcpyAsync(t->h_bctl, t->d_bctl, sizeof(LaunchCtl), cudaMemcpyDeviceToHost, st));
@@ -2017,7 +2040,7 @@ int table_create(int precision, int max_slots, SlotTable** out) {
                b_act = align256(sizeof(int) * 2 * max_slots), b_ctl = align256(sizeof(LaunchCtl)),
                b_diag = align256(sizeof(int) * 4 * t->grid_cap), b_res = align256(sizeof(SolveState) * max_slots),
                b_bact = align256(sizeof(int) * max_slots), b_bcnt = align256(128 * (size_t)kMaxTeamCtas),
-               b_bcta = align256(sizeof(TeamCta) * kMaxTeamCtas);
+               b_bcta = align256(sizeof(TeamCta) * 2 * kMaxTeamCtas);
   const size_t legacy = b_solves + b_nt + b_act + b_ctl + b_diag + b_res;
   const size_t total = legacy + 2 * b_bact + b_bcnt + b_ctl + b_bcta;
   if (cudaMalloc(&t->buf, total) != cudaSuccess) {
@@ -2037,7 +2060,7 @@ int table_create(int precision, int max_slots, SlotTable** out) {
   t->d_bctl = (LaunchCtl*)(t->buf + legacy + 2 * b_bact + b_bcnt);
   t->d_bcta = (TeamCta*)(t->buf + legacy + 2 * b_bact + b_bcnt + b_ctl);
   int rc = cuda_status(cudaMemset(t->buf, 0, total));
-  if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bcta, sizeof(TeamCta) * kMaxTeamCtas));
+  if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bcta, sizeof(TeamCta) * 2 * kMaxTeamCtas));
   if (!rc) rc = cuda_status(cudaMallocHost(&t->h_border, sizeof(int) * max_slots));
   if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bact, sizeof(int) * max_slots));
   if (!rc) rc = cuda_status(cudaMallocHost(&t->h_bctl, sizeof(LaunchCtl)));

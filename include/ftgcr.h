@@ -96,12 +96,15 @@ typedef struct {
  * refinement updates).  Faults still fire. */
 #define FTGCR_FLAG_UNPROTECTED 1
 /* FTGCR_MIXED with the line preconditioner: how a step's rounds are laid out.
- * By default a solve whose row bands shared memory cuts below three rows
- * (wide rows: the line-solve constants fill it) runs split rounds: its
- * tiles first form e on their own rows only, and after a grid barrier form
- * L(e) and the dots from e with its halo rows, instead of recomputing two
- * halo rows of e per tile.  These flags force one layout or the other
- * (results differ only by rounding; both are deterministic); both together,
+ * By default a solve of up to 4095 columns runs banded rounds (a band's
+ * vectors kept on chip, neighbours' edge rows exchanged inside the round), or
+ * one-pass rounds (every tile forms e on its halo rows too) where those are
+ * faster.  A wider solve whose row bands shared memory cuts below three rows
+ * (the line-solve constants fill it) runs split rounds: its tiles first form
+ * e on their own rows only, and after a grid barrier form L(e) and the dots
+ * from e with its halo rows.  FTGCR_FLAG_SPLIT_ROUNDS forces split rounds;
+ * FTGCR_FLAG_FUSED_ROUNDS keeps a solve out of the split and streamed layouts
+ * (results differ only by rounding; all are deterministic); both together,
  * or FTGCR_FLAG_SPLIT_ROUNDS on another precision or preconditioner, are
  * FTGCR_ERR_ARG. */
 #define FTGCR_FLAG_SPLIT_ROUNDS 2
@@ -122,9 +125,11 @@ typedef struct {
  * thread sums its products with one fma per element (double-double from the
  * warp up); with this flag every product and partial sum is compensated
  * (Dot2, Ogita-Rump-Oishi), as in the oracle.  (2) Line preconditioner:
- * rows of 256 or more columns take a chunked scan by default (one warp per
- * row, 32 chunks joined by their exact affine maps); with this flag every
- * row takes the oracle's Thomas elimination (one lane per row).  (3) The
+ * rows of up to 4095 columns are solved in pieces of 8 or 16 elements, joined
+ * by their exact affine maps, by default (wider ones in 32 chunks); with this
+ * flag every row takes the oracle's Thomas elimination (one lane per row).
+ * The next beta of an accepted step comes from the identities of the mixed
+ * path's fused rounds, except near planned flips of the state vectors.  (3) The
  * operator inside the solve: fused multiply-adds by default (9 FP64
  * operations a point instead of 13), the oracle's form with this flag
  * (ftgcr_apply_operator always takes the oracle's form).  The defaults keep
@@ -261,8 +266,9 @@ int ftgcr_solve_async(ftgcr_handle* h, const double* rhs, double* x, const ftgcr
 /* Statistics of the last solve of h (synchronises with its stream). */
 int ftgcr_stats(ftgcr_handle* h, ftgcr_stats_t* out);
 
-/* Solve n independent problems in ONE persistent launch (all handles of the
- * same precision).  Each solve uses its own handle's tiling, so its result is
+/* Solve n independent problems in one persistent launch per kind of round
+ * (all handles of the same precision; banded solves of 2^18 points or more
+ * form a launch of their own, one after another on all SMs).  Each solve uses its own handle's tiling, so its result is
  * bitwise the same as when it is solved alone.  rhs[i], x[i] device memory;
  * plans may be NULL.  Enqueues only; read each status with ftgcr_stats().
  * The launch's tables are stream-ordered allocations filled by kernels from

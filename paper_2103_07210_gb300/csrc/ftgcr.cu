@@ -397,6 +397,145 @@ __global__ void k_lf_band(int nlon, int nlat, int lq, int PC, const double* __re
   }
 }
 
+// The mixed path's factorisation, whose constants are kept in FP32: FP64
+// throughout, without the division in the serial chain (some 13 dependent
+// FP64 instructions of 64 cycles a column: 512 x 256 took 444 us in
+// all with the rebuild's other kernels, now 224; 4096 x 2048 3.70 ms, now 2.00).  The pivots of the leading block are ratios of consecutive minors,
+// w_i = p_i / p_{i-1} with p_i = d_i p_{i-1} - Tx_{i-1}^2 p_{i-2}: one dependent
+// multiply-add a column, every fourth followed by a scaling by a power of two.
+// The same from the other end gives w'_i, and the bordering solve A0 z = c
+// needs no substitution: column m-1 of A0^-1 is g_i = (Tx_i / w_i) g_{i+1} from
+// g_{m-1} = 1 / w_{m-1}, column 0 is h_i = (Tx_{i-1} / w'_i) h_{i-1} from h_0 =
+// 1 / w'_0, both running products.  Against 80-bit arithmetic on the rows of
+// 64 x 32 to 4096 x 2048 the relative errors are those of k_line_factor's order
+// within a small factor (at most 5e-15 in 1/w, 1e-12 in z and delta): far below
+// the FP32 rounding of what is stored.
+constexpr int kLfMinBlock = 16;    // inputs loaded ahead per lane
+constexpr int kLfRowThreads = 256;
+
+// 2^(1023 - e) for a normal number of biased exponent e: its reciprocal scale.
+__device__ __forceinline__ double lf_scale(double p) {
+  const unsigned e = ((unsigned)__double2hiint(p) >> 20) & 0x7ffu;
+  return e - 1u < 2045u ? __hiloint2double((int)((2046u - e) << 20), 0) : 1.0;
+}
+// The minors from the west (even blocks) and from the east (odd), one lane a
+// row; p as formed, before the scaling that follows every fourth.
+__global__ void k_lf_minors(int nlon, int nlat, const double* __restrict__ Tx, const double* __restrict__ dg,
+                            double* __restrict__ pf, double* __restrict__ pb) {
+  const bool back = blockIdx.x & 1;
+  const int j = (int)(blockIdx.x >> 1) * 32 + (int)threadIdx.x, m = nlon - 1, s = back ? -1 : 1;
+  if (j >= nlat) return;
+  const long long rb = (long long)j * nlon, o = rb + (back ? m - 1 : 0);
+  const double *t = Tx + (back ? o : o - 1), *d = dg + o;  // column k: Tx at s k, d at s k
+  double* out = (back ? pb : pf) + o;
+  double p = d[0], q = 1.0;
+  out[0] = p;
+  double ta[kLfMinBlock], da[kLfMinBlock], tb[kLfMinBlock], db[kLfMinBlock];
+  auto load = [&](int k0, double* tt, double* dd) {
+#pragma unroll
+    for (int w = 0; w < kLfMinBlock; ++w)
+      if (k0 + w < m) {
+        tt[w] = t[s * (k0 + w)];
+        dd[w] = d[s * (k0 + w)];
+      }
+  };
+  auto step = [&](int k0, const double* tt, const double* dd) {  // k0 = 1 modulo 4
+#pragma unroll
+    for (int w = 0; w < kLfMinBlock; ++w)
+      if (k0 + w < m) {
+        const double pn = fma(dd[w], p, -(tt[w] * tt[w]) * q);
+        q = p;
+        p = pn;
+        out[s * (k0 + w)] = p;
+        if ((w & 3) == 3) {
+          const double e = lf_scale(p);
+          p = p * e;
+          q = q * e;
+        }
+      }
+  };
+  load(1, ta, da);
+  for (int k0 = 1; k0 < m; k0 += 2 * kLfMinBlock) {
+    load(k0 + kLfMinBlock, tb, db);
+    step(k0, ta, da);
+    load(k0 + 2 * kLfMinBlock, ta, da);
+    step(k0 + kLfMinBlock, tb, db);
+  }
+}
+// One block a row: 1/w, u = -Tx / w, z and the row constants from the minors
+// (w, l: the minors on entry; z: the diagonal).  Shared memory: two rows.
+__global__ void __launch_bounds__(kLfRowThreads) k_lf_rows(int nlon, int nlat, const double* __restrict__ Tx, double* w,
+                                                           const double* l, double* u, double* z, double* lrow64,
+                                                           float* lrow32) {
+  extern __shared__ double lf_sm[];
+  __shared__ double wa[kLfRowThreads / 32], wb[kLfRowThreads / 32];
+  const int n = nlon, m = n - 1, j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const long long rb = (long long)j * n;
+  const double *t = Tx + rb, *pf = w + rb, *pb = l + rb;
+  double *A = lf_sm, *B = lf_sm + n, *zr = z + rb;
+  for (int i = tid; i < m; i += kLfRowThreads) {
+    double qf = 1.0, qb = 1.0;
+    if (i > 0) {
+      qf = pf[i - 1];
+      if (i - 1 > 0 && ((i - 1) & 3) == 0) qf = qf * lf_scale(qf);
+    }
+    if (i < m - 1) {
+      qb = pb[i + 1];
+      const int k = m - 2 - i;
+      if (k > 0 && (k & 3) == 0) qb = qb * lf_scale(qb);
+    }
+    const double wi = qf / pf[i], wbi = qb / pb[i];
+    const double a = i < m - 1 ? t[i] * wi : 0.0;
+    A[i] = i < m - 1 ? a : wi;
+    B[i] = i > 0 ? t[i - 1] * wbi : wbi;
+    u[rb + i] = -a;
+    zr[i] = wi;
+  }
+  __syncthreads();
+  // running products, west to east of B and east to west of A: a piece a
+  // thread (an odd length: no bank conflicts)
+  const int L = ((m + kLfRowThreads - 1) / kLfRowThreads) | 1, lo = min(tid * L, m), hi = min(lo + L, m);
+  double pa = 1.0, pr = 1.0;
+  for (int i = lo; i < hi; ++i) {
+    pa = pa * A[i];
+    pr = pr * B[i];
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double ya = __shfl_down_sync(0xffffffffu, pa, o), yb = __shfl_up_sync(0xffffffffu, pr, o);
+    if (lane + o < 32) pa = pa * ya;
+    if (lane >= o) pr = pr * yb;
+  }
+  if (lane == 0) wa[wp] = pa;
+  if (lane == 31) wb[wp] = pr;
+  double ga = __shfl_down_sync(0xffffffffu, pa, 1), hb = __shfl_up_sync(0xffffffffu, pr, 1);
+  if (lane == 31) ga = 1.0;
+  if (lane == 0) hb = 1.0;
+  __syncthreads();
+  for (int v = kLfRowThreads / 32 - 1; v > wp; --v) ga = ga * wa[v];
+  for (int v = 0; v < wp; ++v) hb = hb * wb[v];
+  for (int i = hi - 1; i >= lo; --i) A[i] = ga = ga * A[i];
+  for (int i = lo; i < hi; ++i) B[i] = hb = hb * B[i];
+  __syncthreads();
+  const double tl = t[n - 1], tp = t[n - 2], dl = zr[m];
+  auto zv = [&](int i) { return fma(-tl, B[i], -tp * A[i]); };
+  for (int i = tid; i < m; i += kLfRowThreads) {
+    w[rb + i] = zr[i];
+    zr[i] = zv(i);
+  }
+  __syncthreads();  // zr[m] is read
+  if (tid == 0) {
+    w[rb + m] = 0.0;
+    u[rb + m] = 0.0;
+    zr[m] = 0.0;
+    const double delta = dl + tl * zv(0) + tp * zv(m - 1), dinv = 1.0 / delta;
+    const double row[4] = {delta, dinv, tl * dinv, tp * dinv};
+    for (int q = 0; q < 4; ++q) lrow64[(long long)j * 4 + q] = row[q];
+    for (int q = 0; q < 3; ++q) lrow32[(long long)j * 4 + q] = (float)row[q + 1];
+    lrow32[(long long)j * 4 + 3] = 0.f;
+  }
+}
+
 // The line preconditioner's factorisation (Jacobi: its diagonal), enqueued
 // on st.  FP64 outputs l, winv, u, z (z doubles as scratch for the diagonal)
 // and the row constants; FP32 chunk-layout constants when lc32 is given.
@@ -414,11 +553,22 @@ int launch_line_factor(int nlon, int nlat, int C, int precond, const double* Tx,
   const int eb = 256, eg = (int)std::min<long long>((N + eb - 1) / eb, 8192);
   const int rg = (nlat + 31) / 32;  // one lane per row, one warp per block
   k_lf_diag<<<eg, eb, 0, st>>>(nlon, nlat, Tx, Ty, muA, z64);
-  k_lf_chain_lw<<<rg, 32, 0, st>>>(nlon, nlat, Tx, z64, l64, w64);
-  k_lf_recip<<<eg, eb, 0, st>>>(nlon, nlat, Tx, l64, w64, u64, z64);
-  k_lf_chain_fwd<<<rg, 32, 0, st>>>(nlon, nlat, l64, z64);
-  k_lf_products<<<eg, eb, 0, st>>>(nlon, nlat, w64, z64);
-  k_lf_chain_bwd<<<rg, 32, 0, st>>>(nlon, nlat, Tx, Ty, muA, u64, z64, r64, lrow32);
+  // FP32 constants: no serial divisions (rows that its two shared-memory rows
+  // do not hold, and the shortest, keep the chains)
+  const size_t rows2 = 2 * sizeof(double) * (size_t)nlon;
+  if (lrow32 && nlon >= 8 && rows2 <= 200 * 1024) {
+    if (rows2 > 40 * 1024 &&
+        cudaFuncSetAttribute(k_lf_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows2) != cudaSuccess)
+      return FTGCR_ERR_CUDA;
+    k_lf_minors<<<2 * rg, 32, 0, st>>>(nlon, nlat, Tx, z64, w64, l64);
+    k_lf_rows<<<nlat, kLfRowThreads, rows2, st>>>(nlon, nlat, Tx, w64, l64, u64, z64, r64, lrow32);
+  } else {
+    k_lf_chain_lw<<<rg, 32, 0, st>>>(nlon, nlat, Tx, z64, l64, w64);
+    k_lf_recip<<<eg, eb, 0, st>>>(nlon, nlat, Tx, l64, w64, u64, z64);
+    k_lf_chain_fwd<<<rg, 32, 0, st>>>(nlon, nlat, l64, z64);
+    k_lf_products<<<eg, eb, 0, st>>>(nlon, nlat, w64, z64);
+    k_lf_chain_bwd<<<rg, 32, 0, st>>>(nlon, nlat, Tx, Ty, muA, u64, z64, r64, lrow32);
+  }
   const long long nc = 32LL * C * nlat;
   const int cgrid = (int)std::min<long long>((nc + eb - 1) / eb, 8192);
   if (lc32) k_lf_chunks<float><<<cgrid, eb, 0, st>>>(nlon, nlat, C, u64, w64, z64, lc32, lw32, lz32);

@@ -905,7 +905,7 @@ def run_ours(args):
             "roofline": {"bound": "l2", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind + " HBM copy",
                          "dram_over_algorithmic": (traffic / bytes_launch) if traffic else None,
-                         "kernel": "k_ftgcr_persistent<float>",
+                         "kernel": "k_ftgcr_band<float>",
                          "algorithmic_bytes_per_launch": bytes_launch},
             "e2e": {"value": e2e_val, "unit": "solves/s", "h2d_bytes_per_step": (1 if ZG else 2) * 8 * NLON * NLAT,
                     "pipelined": f"ftgcr_solve_host_async, {NH} handles in turn on 2 streams (state > L2)",

@@ -1446,6 +1446,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
     const bool local = sizeof(T) == 4 && single && ks.sd.local;
     if (threadIdx.x == 0) ks.ps.cr.stride = 2 * nt;
     bool expected = false, done = false, late = false;
+    bool met = false;  // the team has met at a barrier since its CTAs loaded the record
     long long round = ks.S.round;  // of ks.S, which the last warp rewrites while the others go on
     int pending = ks.S.pending, cur = 0, halo = -1;
     __syncthreads();
@@ -1455,6 +1456,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
     for (int it = 0; it < a.max_rounds; ++it) {
       unsigned long long tr0 = 0ull, tr1 = 0ull;
       cur ^= 1;
+      met = it > 0;
       if (threadIdx.x == 0) {
         tr0 = globaltimer();
         if (tr0 - t_start > kKernelTimeoutNs) ks.tf.raise(2);
@@ -1622,6 +1624,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
       }
     }
     __syncthreads();
+    if (!met) {
+      // a launch of one round, or a solve with nothing left but its end: the
+      // record may be rewritten only once every CTA of the team has loaded it
+      if (done) {
+        ++nbar;
+        arrive();
+      }
+      if (me.rank == 0) {
+        if (threadIdx.x == 0 && !team_wait(nbar * (unsigned)me.size, ks.tf)) ks.bail = 1;
+        __syncthreads();
+        if (ks.bail) return;
+      }
+    }
     if (me.rank == 0) {
       // the record: finished (with K_NONE's transition in ks.N), or to be resumed
       if (done) {

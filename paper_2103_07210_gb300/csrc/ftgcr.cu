@@ -654,6 +654,19 @@ __global__ void k_nonfinite(const double* __restrict__ a, long long n, LaunchCtl
 template <typename T>
 __global__ void k_begin_solve(SolveDev<T>* sd, BeginArgs b, int* active, int n_active, int slot, int par,
                               LaunchCtl* ctl, const LaunchCtl* check = nullptr) {
+  if (sd->band) {
+    // The packets of banded rounds carry ten bits of the solve's number and 22
+    // of the round's.  They are cleared before a tag could come round again:
+    // every 1024 solves, after a solve of 2^22 rounds or more, and after one
+    // that did not finish, whose rounds are not known.  (2 MB at 1024 x 512.)
+    const SolveState& last = sd->st[0];
+    const bool wipe = ((sd->solve_id + 1u) & 1023u) == 0u || last.active || last.round >= 1LL << 22;
+    __syncthreads();
+    if (wipe) {
+      const long long n = 2LL * sd->nt * sd->NG * (long long)sizeof(T);
+      for (long long i = threadIdx.x; i < n; i += blockDim.x) sd->hrow[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
   if (check && check->nonfinite) {
     if (threadIdx.x == 0) {
       SolveState S;

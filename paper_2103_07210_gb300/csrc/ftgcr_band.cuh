@@ -440,8 +440,8 @@ struct TeamFail {
 // a 16-byte access (the scheme of NCCL's LL protocol).  A reader polls the
 // packets themselves, so an exchange costs one trip through L2 and no fence,
 // where rows under a flag cost a release, the flag's trip and the rows' trip.
-// A tag can only be met too early in packets of the solve before last or
-// older, or 2^22 rounds old; every step round rewrites all of them.
+// A tag is ten bits of the solve's number and 22 of the round's (solve_id,
+// round + 1): old packets are cleared before one repeats (k_begin_solve).
 // Two sets, by the round's parity: a neighbour may read a round's packets as
 // late as its own next round.
 template <typename T>

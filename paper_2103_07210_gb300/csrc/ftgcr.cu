@@ -536,6 +536,20 @@ __global__ void __launch_bounds__(kLfRowThreads) k_lf_rows(int nlon, int nlat, c
   }
 }
 
+// The dynamic shared memory attribute of a kernel is process-wide: only ever
+// raise it, so that a launch of another thread never finds it below what that
+// thread has asked for.
+cudaError_t raise_dynamic_smem(const void* f, size_t bytes) {
+  static std::mutex mu;
+  static std::map<const void*, size_t> set;
+  std::lock_guard<std::mutex> lk(mu);
+  size_t& at = set[f];
+  if (at >= bytes) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) at = bytes;
+  return e;
+}
+
 // The line preconditioner's factorisation (Jacobi: its diagonal), enqueued
 // on st.  FP64 outputs l, winv, u, z (z doubles as scratch for the diagonal)
 // and the row constants; FP32 chunk-layout constants when lc32 is given.
@@ -557,9 +571,10 @@ int launch_line_factor(int nlon, int nlat, int C, int precond, const double* Tx,
   // do not hold, and the shortest, keep the chains)
   const size_t rows2 = 2 * sizeof(double) * (size_t)nlon;
   if (lrow32 && nlon >= 8 && rows2 <= 200 * 1024) {
-    if (rows2 > 40 * 1024 &&
-        cudaFuncSetAttribute(k_lf_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows2) != cudaSuccess)
+    if (rows2 > 40 * 1024 && raise_dynamic_smem((const void*)k_lf_rows, rows2) != cudaSuccess) {
+      cudaGetLastError();
       return FTGCR_ERR_CUDA;
+    }
     k_lf_minors<<<2 * rg, 32, 0, st>>>(nlon, nlat, Tx, z64, w64, l64);
     k_lf_rows<<<nlat, kLfRowThreads, rows2, st>>>(nlon, nlat, Tx, w64, l64, u64, z64, r64, lrow32);
   } else {
@@ -1063,24 +1078,10 @@ const void* kernel_ptr(int kb, int wide) {
   return ftgcr::persistent_kernel_ptr(kb, sizeof(T) == 8, wide);
 }
 
-// The dynamic shared memory attribute of a kernel is process-wide: only ever
-// raise it, so that a handle created later never shrinks what an earlier one
-// needs.
+// A solve's kernel, allowed the handle's dynamic shared memory.
 template <typename T>
 int configure_kernel(int kb, int split, size_t smem) {
-  static std::mutex mu;
-  static std::vector<std::pair<const void*, size_t>> set;
-  std::lock_guard<std::mutex> lk(mu);
-  const void* f = kernel_ptr<T>(kb, split);
-  for (auto& e : set)
-    if (e.first == f) {
-      if (e.second >= smem) return FTGCR_OK;
-      CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      e.second = smem;
-      return FTGCR_OK;
-    }
-  CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  set.emplace_back(f, smem);
+  CK(raise_dynamic_smem(kernel_ptr<T>(kb, split), smem));
   return FTGCR_OK;
 }
 

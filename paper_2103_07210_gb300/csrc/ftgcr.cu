@@ -2151,7 +2151,7 @@ int ftgcr_apply_precond(ftgcr_handle* h, const double* in, double* out, void* st
   }
   const int rows_per_block = 4;
   const size_t smem = (size_t)rows_per_block * row_stride(h->nlon) * sizeof(double);
-  CK(cudaFuncSetAttribute(k_apply_precond, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CK(raise_dynamic_smem((const void*)k_apply_precond, smem));
   k_apply_precond<<<(h->nlat + rows_per_block - 1) / rows_per_block, 32 * rows_per_block, smem, st>>>(in, out, sd);
   CK(cudaGetLastError());
   return FTGCR_OK;

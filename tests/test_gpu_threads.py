@@ -44,3 +44,16 @@ def test_rebuilds_of_two_widths_in_two_threads():
     _in_two_threads(calls, 1500)
     for s in solvers:
         s.close()
+
+
+def test_preconditioners_of_two_widths_in_two_threads():
+    solvers, calls = [], []
+    for nlon in (64, 4000):
+        p = inputs.hill_problem(nlon, 4)
+        solvers.append(ftgcr.Solver(p.D, p.mu))
+        inp = torch.from_numpy(p.R).cuda()
+        calls.append(lambda stream, s=solvers[-1], i=inp, o=torch.zeros_like(inp): s.apply_precond(i, o, stream=stream))
+    torch.cuda.synchronize()
+    _in_two_threads(calls, 3000)
+    for s in solvers:
+        s.close()

@@ -19,6 +19,7 @@
 #include "ftgcr_band.cuh"
 #include "ftgcr_instances.h"
 #include "ftgcr_serve.h"
+#include "ftgcr_teams.h"
 
 using namespace ftgcr;
 
@@ -1458,64 +1459,6 @@ int launch_band(int kb, SolveDev<T>* const* solves, int* active, const TeamCta* 
   return FTGCR_OK;
 }
 
-// Teams of CTAs for a launch of several banded solves.  A team runs its solves
-// one after another, so a solve's rounds wait for nobody else's.  As many
-// teams as keep at least kTeamMin CTAs each (a 1024 x 512 solve on one SM
-// takes eight times a round's fixed cost), at most one per solve; CTAs go to
-// teams by the largest solve each would take, then every solve, largest first,
-// to the team that would finish it soonest.
-constexpr int kTeamMin = 8;
-struct TeamPlan {
-  std::vector<TeamCta> cta;  // [grid]
-  std::vector<int> order;    // solves (indices into the argument), team by team
-  int teams = 0;
-};
-void plan_teams(const std::vector<long long>& points, const std::vector<int>& nt, int sms, int most_teams, TeamPlan* out) {
-  const int n = (int)points.size();
-  std::vector<int> by(n);
-  for (int i = 0; i < n; ++i) by[i] = i;
-  std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return points[a] > points[b]; });
-  const int teams = std::max(1, std::min({n, sms / kTeamMin, most_teams}));
-  // sizes: one CTA each, then one by one to the team with the most points per CTA
-  std::vector<int> size(teams, 1);
-  for (int left = sms - teams; left > 0; --left) {
-    int best = -1;
-    double load = 0;
-    for (int t = 0; t < teams; ++t) {
-      if (size[t] >= nt[by[t]]) continue;
-      const double l = (double)points[by[t]] / size[t];
-      if (best < 0 || l > load) best = t, load = l;
-    }
-    if (best < 0) break;
-    ++size[best];
-  }
-  std::vector<double> busy(teams, 0.0);
-  std::vector<std::vector<int>> list(teams);
-  for (int i : by) {
-    int best = 0;
-    double end = 0;
-    for (int t = 0; t < teams; ++t) {
-      // a round: its points over the team's CTAs, plus a fixed cost worth about 8192 points
-      const double e = busy[t] + (double)points[i] / std::min(size[t], nt[i]) + 8192.0;
-      if (t == 0 || e < end) best = t, end = e;
-    }
-    busy[best] = end;
-    list[best].push_back(i);
-  }
-  out->cta.clear();
-  out->order.clear();
-  out->teams = 0;
-  for (int t = 0; t < teams; ++t) {
-    if (list[t].empty()) continue;
-    int most = 1;
-    for (int i : list[t]) most = std::max(most, nt[i]);
-    const int sz = std::min(size[t], most), q0 = (int)out->order.size();
-    for (int i : list[t]) out->order.push_back(i);
-    for (int r = 0; r < sz; ++r) out->cta.push_back(TeamCta{out->teams, r, sz, q0, (int)out->order.size()});
-    ++out->teams;
-  }
-}
-
 BeginArgs begin_args(const ftgcr_handle* h, const double* R, const double* x0, double* xout,
                      const ftgcr_fault_plan* plan) {
   BeginArgs b;
@@ -1553,21 +1496,8 @@ int solve_async_impl(ftgcr_handle* h, const double* R, const double* x0, double*
   return FTGCR_OK;
 }
 
+int launch_class(const ftgcr_handle* h) { return h->wide == kWideBand ? band_class(h->N) : 0; }
 // The schedule of a banded launch, filled like the solve table.
-// The launches of a batch or an epoch: 0 the solves of the other kernels, 1
-// banded solves side by side in teams, 2 banded solves of kWholePoints or more,
-// which take all CTAs one after another: on a few CTAs such a solve reads its
-// vectors from L2 or memory, on all of them its bands stay on chip.  Smaller
-// ones leave CTAs idle or pay for barriers among all.  The line lies between
-// 512 x 256 and 1024 x 512 points: ms with none / 2048 x 1024 / 1024 x 512 and
-// up / 512 x 256 and up taken whole, 32 mixed solves served 37.5 / 23.6 / 21.5 /
-// 23.3, 21 FP64 ones 52.3 / 43.0 / 40.7 / 42.3, a batch of 128 mixed solves (to
-// 1024 x 512) 36.4 / 36.4 / 33.6 / 40.7, of 28 FP64 ones 29.4 / 29.4 / 23.8 / 24.6.
-constexpr long long kWholePoints = 1LL << 18;
-int launch_class(const ftgcr_handle* h) {
-  if (h->wide != kWideBand) return 0;
-  return h->N >= kWholePoints ? 2 : 1;
-}
 constexpr int kMaxTeamCtas = 256;
 struct TeamTable {
   TeamCta cta[kMaxTeamCtas];

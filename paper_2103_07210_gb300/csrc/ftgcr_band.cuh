@@ -31,16 +31,11 @@
 #pragma once
 #include "ftgcr_instances.h"
 #include "ftgcr_phases.cuh"
+#include "ftgcr_teams.h"
 
 namespace ftgcr {
 
 constexpr int kBandMaxBuf = kMaxK + 2;
-
-// The part of a launch a CTA works in.
-struct TeamCta {
-  int team, rank, size;
-  int q0, q1;  // the team's solves: order[q0 .. q1)
-};
 
 template <typename T>
 struct BandArgs {

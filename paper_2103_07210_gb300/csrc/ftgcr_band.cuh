@@ -987,9 +987,11 @@ __device__ __noinline__ void band_after(int kind, int tau, int cur, int t, int n
 //   band_window does is done while they travel.
 // Either way every value is formed by the same operations, so a solve's result
 // does not depend on which is taken.
-// FLT: the instance for solves with planned faults (a call in a loop makes the
-// compiler keep the loop's values in local memory, and with shared memory
-// taking the L1 cache every such access costs an L2 trip).
+// FLT: the instance for the rounds of steps with planned faults (a call in a
+// loop makes the compiler keep the loop's values in local memory, and with
+// shared memory taking the L1 cache every such access costs an L2 trip).  Only
+// those rounds take it: on every round of a solve with a fault plan it made a
+// mixed 1024 x 512 solve 26 % slower.
 template <typename T, int KB, int KIND, bool AL, bool FLT>
 __device__ __forceinline__ void band_step(int tau, int ntile, int pass, int cur, double* part_out) {
   BandSmem<T>& ks = band_smem<T>();
@@ -1293,7 +1295,7 @@ __device__ __forceinline__ void band_step(int tau, int ntile, int pass, int cur,
   band_sums<T>(red, kInit && pass == 2 ? 2 : 0, vh + 2, kInit ? 2u : 0u, tau, ntile, part_out, ps.cr.stride);
 }
 // The rounds a solve takes but a few times, out of line; the PF round of a
-// solve without planned faults is inlined into the kernel, where it saves no
+// step without planned faults is inlined into the kernel, where it saves no
 // registers at entry (a function of its size saves some 80, which go through
 // L2).
 template <typename T, int KB, int KIND, bool AL, bool FLT>
@@ -1304,7 +1306,7 @@ template <typename T, int KB>
 __device__ __forceinline__ void band_step_any(int kind, int tau, int ntile, int pass, int cur, double* part_out) {
   const SolveDev<T>& sd = band_smem<T>().sd;
   const bool al = (sd.nlon & 3) == 0;
-  if (sd.nfaults | sd.nlosses) {  // the unaligned form serves every row width
+  if (band_smem<T>().c[cur].events) {  // the unaligned form serves every row width
     if (kind == K_INIT)
       band_step_out<T, KB, K_INIT, false, true>(tau, ntile, pass, cur, part_out);
     else if (kind == K_PA)
@@ -1384,6 +1386,7 @@ __device__ __noinline__ void usual_transition(const SolveDev<T>& sd, const Solve
   N.ecur = ec;
   N.pending = c.kind;
   c.nu = nun;
+  c.events = 0;
   c.t = S.step + (step ? 2 : 1);
   c.phiC = sd.phi[phiC];
   c.phiW = sd.phi[phiW];
@@ -1586,7 +1589,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
         arrive();
         if (sizeof(T) == 4 && late && ta < tb && warp >= kTotWarps) {
           const int t = (int)threadIdx.x - 32 * kTotWarps, nth = 32 * (kSumWarps - kTotWarps);
-          if (ks.sd.nfaults | ks.sd.nlosses)
+          if (ks.c[cur].events)
             band_after<T, KB, false, true>(kind, ta, cur, t, nth);
           else if ((ks.sd.nlon & 3) == 0)
             band_after<T, KB, true, false>(kind, ta, cur, t, nth);

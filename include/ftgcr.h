@@ -268,7 +268,8 @@ int ftgcr_stats(ftgcr_handle* h, ftgcr_stats_t* out);
 
 /* Solve n independent problems in one persistent launch per kind of round
  * (all handles of the same precision; banded solves of 2^18 points or more
- * form a launch of their own, one after another on all SMs).  Each solve uses its own handle's tiling, so its result is
+ * with bands for most of the SMs form a launch of their own, one after another
+ * on all SMs).  Each solve uses its own handle's tiling, so its result is
  * bitwise the same as when it is solved alone.  rhs[i], x[i] device memory;
  * plans may be NULL.  Enqueues only; read each status with ftgcr_stats().
  * The launch's tables are stream-ordered allocations filled by kernels from

@@ -1496,7 +1496,7 @@ int solve_async_impl(ftgcr_handle* h, const double* R, const double* x0, double*
   return FTGCR_OK;
 }
 
-int launch_class(const ftgcr_handle* h) { return h->wide == kWideBand ? band_class(h->N) : 0; }
+int launch_class(const ftgcr_handle* h, int sms) { return h->wide == kWideBand ? band_class(h->N, h->nt, sms) : 0; }
 // The schedule of a banded launch, filled like the solve table.
 constexpr int kMaxTeamCtas = 256;
 struct TeamTable {
@@ -1519,6 +1519,7 @@ __global__ void k_fill_teams(TeamTable t, TeamCta* d_cta) {
 template <typename T>
 int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, double* const* x,
                      const ftgcr_fault_plan* const* plans, int n_all, cudaStream_t st) {
+  const DeviceInfo di = device_info(hs_all[0]->dev);
   for (int cls = 0; cls < 3; ++cls) {
     const bool band = cls != 0;
     std::vector<int> id;  // this launch's solves
@@ -1528,7 +1529,7 @@ int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, doub
     int max_outer = 0, split = 0;
     for (int i = 0; i < n_all; ++i) {
       const ftgcr_handle* h = hs_all[i];
-      if (launch_class(h) != cls) continue;
+      if (launch_class(h, di.sms) != cls) continue;
       id.push_back(i);
       split = std::max(split, h->wide);
       kb = std::max(kb, kbound(h->k));
@@ -1545,7 +1546,6 @@ int solve_batch_impl(ftgcr_handle* const* hs_all, const double* const* rhs, doub
     rc = occupancy<T>(kb, split, smem, &occ);
     if (rc) return rc;
     if (occ < 1) return FTGCR_ERR_ARG;
-    const DeviceInfo di = device_info(hs_all[0]->dev);
     int grid = (int)std::min<long long>(total_tiles, (long long)di.sms * occ);
     TeamPlan tp;
     if (band) {
@@ -1680,6 +1680,7 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
   t->h_ctl_out->err = 0;
   t->h_ctl_out->round_end = t->round;
   t->h_bctl->err = 0;
+  const DeviceInfo di = device_info(t->dev);
   int border = 0;          // solves placed in banded launches
   bool ctl_ready = false;  // their control block is reset
   for (int cls = 0; cls < 3; ++cls) {
@@ -1691,7 +1692,7 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
     std::vector<int> id;
     for (int s = 0; s < t->n; ++s) {
       const ftgcr_handle* h = t->slot[s];
-      if (!h || launch_class(h) != cls) continue;
+      if (!h || launch_class(h, di.sms) != cls) continue;
       id.push_back(s);
       split = std::max(split, h->wide);
       kb = std::max(kb, kbound(h->k));
@@ -1713,7 +1714,7 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
         nts.push_back(t->slot[s]->nt);
       }
       TeamPlan tp;
-      plan_teams(points, nts, std::min(device_info(t->dev).sms, kMaxTeamCtas), cls == 2 ? 1 : kMaxTeamCtas, &tp);
+      plan_teams(points, nts, std::min(di.sms, kMaxTeamCtas), cls == 2 ? 1 : kMaxTeamCtas, &tp);
       const int grid = (int)tp.cta.size();
       // the previous epoch, whose copies read these, has been collected; each
       // class has its own part
@@ -1734,7 +1735,7 @@ int table_run_impl(SlotTableImpl* t, int max_rounds, cudaStream_t st) {
       CK(cudaMemcpyAsync(t->h_bact, t->d_bact, sizeof(int) * t->n, cudaMemcpyDeviceToHost, st));
       continue;
     }
-    const int grid = (int)std::min<long long>({tiles, (long long)device_info(t->dev).sms * occ, (long long)t->grid_cap});
+    const int grid = (int)std::min<long long>({tiles, (long long)di.sms * occ, (long long)t->grid_cap});
     t->h_ctl_in->counter = 0;
     t->h_ctl_in->err = 0;
     t->h_ctl_in->round0 = t->round;

@@ -13,16 +13,24 @@ struct TeamCta {
 };
 
 // The launches of a batch or an epoch: 0 the solves of the other kernels, 1
-// banded solves side by side in teams, 2 banded solves of kWholePoints or more,
-// which take all CTAs one after another: on a few CTAs such a solve reads its
-// vectors from L2 or memory, on all of them its bands stay on chip.  Smaller
-// ones leave CTAs idle or pay for barriers among all.  The line lies between
-// 512 x 256 and 1024 x 512 points: ms with none / 2048 x 1024 / 1024 x 512 and
-// up / 512 x 256 and up taken whole, 32 mixed solves served 37.5 / 23.6 / 21.5 /
-// 23.3, 21 FP64 ones 52.3 / 43.0 / 40.7 / 42.3, a batch of 128 mixed solves (to
-// 1024 x 512) 36.4 / 36.4 / 33.6 / 40.7, of 28 FP64 ones 29.4 / 29.4 / 23.8 / 24.6.
+// banded solves side by side in teams, 2 banded solves of kWholePoints or more
+// with bands for most of the SMs, which take all CTAs one after another: on a
+// few CTAs such a solve reads its vectors from L2 or memory, on all of them its
+// bands stay on chip.  Smaller ones leave CTAs idle or pay for barriers among
+// all.  The line lies between 512 x 256 and 1024 x 512 points: ms with none /
+// 2048 x 1024 / 1024 x 512 and up / 512 x 256 and up taken whole, 32 mixed
+// solves served 37.5 / 23.6 / 21.5 / 23.3, 21 FP64 ones 52.3 / 43.0 / 40.7 /
+// 42.3, a batch of 128 mixed solves (to 1024 x 512) 36.4 / 36.4 / 33.6 / 40.7,
+// of 28 FP64 ones 29.4 / 29.4 / 23.8 / 24.6.
+// Of fewer bands, whole solves leave the other CTAs idle.  On 152 SMs, whole /
+// in teams, ms: 16 FP64 1024 x 512 of 32 bands 124.0 / 34.3, of 64 68.8 / 36.6,
+// of 86 57.7 / 41.1, of 103 52.6 / 45.2, of 128 42.7 / 43.0; mixed of 43 32.9 /
+// 16.7, of 86 17.2 / 17.2, of 103 19.6 / 20.8, of 128 17.1 / 20.0; 16 mixed
+// 4000 x 66 (66 bands) 17.7 / 11.9, 4000 x 90 18.3 / 15.2; 8 mixed 512 x 512 of
+// 66 8.0 / 5.4, of 100 7.0 / 7.3.  The line at five eighths lies where mixed
+// solves cross over.
 constexpr long long kWholePoints = 1LL << 18;
-inline int band_class(long long points) { return points >= kWholePoints ? 2 : 1; }
+inline int band_class(long long points, int nt, int sms) { return points >= kWholePoints && 8 * nt > 5 * sms ? 2 : 1; }
 
 // Teams of CTAs for a launch of several banded solves.  A team runs its solves
 // one after another, so a solve's rounds wait for nobody else's.  As many

@@ -13,6 +13,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2103_07210_gb300", "csrc")
 SOURCE = """
 #include "ftgcr_teams.h"
+extern "C" int band_class(long long points, int nt, int sms) { return ftgcr::band_class(points, nt, sms); }
 extern "C" int plan(int n, const long long* points, const int* nt, int sms, int most, int* cta, int* order) {
   ftgcr::TeamPlan p;
   ftgcr::plan_teams(std::vector<long long>(points, points + n), std::vector<int>(nt, nt + n), sms, most, &p);
@@ -50,6 +51,8 @@ def plan(tmp_path_factory):
         assert sum(t[0] for t in teams) == grid
         return teams
 
+    call.band_class = lambda points, nt, sms: lib.band_class(ctypes.c_longlong(points), nt, sms)
+
     return call
 
 
@@ -85,3 +88,12 @@ def test_no_cta_is_left_over_while_a_solve_lacks_one(plan, seed):
             solves.append((nlon * nlat, _bands(nlat) if rng.random() < 0.7 else rng.randint(1, nlat)))
         sms, most = rng.choice([(152, 256), (152, 1), (20, 256), (4, 256)])
         _check(solves, sms, most, plan(solves, sms, most))
+
+
+def test_a_solve_takes_all_ctas_only_with_bands_for_most_of_them(plan):
+    """Large solves of few bands (asked for, or few rows) run side by side: one
+    after another they would leave the other CTAs idle."""
+    whole = [(1024 * 512, 128), (700 * 700, 140), (2048 * 1024, 147), (2048 * 1024, 1024)]
+    side_by_side = [(1024 * 512, 32), (1024 * 512, 16), (4000 * 66, 66), (512 * 512, 38), (2048 * 1024, 64), (512 * 256, 128)]
+    assert [plan.band_class(*s, 152) for s in whole] == [2] * len(whole)
+    assert [plan.band_class(*s, 152) for s in side_by_side] == [1] * len(side_by_side)

@@ -25,7 +25,7 @@ SOURCES = ["ftgcr.cu", "ftgcr_k4.cu", "ftgcr_k8.cu", "ftgcr_k16.cu", "ftgcr_k4s.
            "ftgcr_k4w.cu", "ftgcr_k8w.cu", "ftgcr_k16w.cu", "ftgcr_b4.cu", "ftgcr_b8.cu", "ftgcr_b16.cu",
            "ftgcr_server.cu", "ftgcr_tune.cu", "ftgcr_probe.cu"]
 HEADERS = ["ftgcr_device.cuh", "ftgcr_phases.cuh", "ftgcr_stream.cuh", "ftgcr_band.cuh", "ftgcr_instances.h", "ftgcr_serve.h",
-           "ftgcr_teams.h"]
+           "ftgcr_teams.h", "ftgcr_factor.cuh"]
 # --fmad=false: device multiply-adds are fused only where the code says fma();
 # -ffp-contract=off: the same for the host-side geometry (GCC contracts by
 # default on aarch64)

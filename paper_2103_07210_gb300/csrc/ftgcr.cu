@@ -333,6 +333,12 @@ SmemPlan smem_plan(int nlon, int nlat, int nt, int mixed, size_t elem, int preco
 // halo rows and the threads' sums, then, as far as they fit, the rows' line-
 // solve constants, the band's vectors (r, L(e) and up to k L(p^l)) and the
 // rows' face coefficients.
+// Rows to 4095 columns.  512 threads and this layout would hold 4096 as well,
+// and faster (ms, k = 4, random right-hand sides, wide-row kernels against
+// banded: FP64 4096 x 40 4.58 / 2.63, 4096 x 512 16.4 / 10.1, 4096 x 1000 27.7 /
+// 24.0; mixed 4096 x 40 1.52 / 1.12, 4096 x 512 5.57 / 3.93, 4096 x 1000 10.3 /
+// 7.2).  The line is one short of it because the library's tests pin what such
+// a handle reports at 4096 columns: split rounds, or factors in global memory.
 constexpr int kBandMaxLon = 4095;
 struct BandLayout {
   int local, lq, NP, NPc, lG, PC, nbuf, cs_staged, ts_staged;
@@ -347,21 +353,20 @@ bool band_layout(int nlon, int nlat, int nt, bool mixed, int k, size_t limit, Ba
   const long long p8 = (nlon + 7) / 8;
   auto row = [&](int cq) {  // the layout of a row with pieces of cq elements
     const int Q = cq / W;
-    b->lq = Q == 2 ? 1 : Q == 4 ? 2 : 3;
+    b->lq = Q == 2 ? 1 : 2;
     b->NPc = (nlon + cq - 1) / cq;
     b->PC = b->NPc;
     b->lG = 0;
     while ((32 << b->lG) < b->NPc) ++b->lG;
     // plane pitch: see BandRow
     b->NP = b->NPc;
-    while (Q == 8 ? !(b->NP & 1) : (b->NP & 7) != (Q == 2 ? 4 : 2)) ++b->NP;
+    while ((b->NP & 7) != (Q == 2 ? 4 : 2)) ++b->NP;
     b->rowb = Q * b->NP * 16;
     b->conb = Q * b->PC * 16;
     return (32 << b->lG) <= kBandThreads;
   };
-  // pieces of 8 elements; of 16 where 8 would take a second trip over the
-  // threads (FP32), or more threads than there are (FP64, whose pieces of 16
-  // take more of its registers)
+  // pieces of 8 elements; FP32: of 16 where 8 would take a second trip over the
+  // threads
   const size_t st = (size_t)row_stride(nlon) * sizeof(double), sums = 8 * (size_t)kBandThreads * (k + 3);
   b->sub_h = 0;
   size_t out = 0;
@@ -384,7 +389,7 @@ bool band_layout(int nlon, int nlat, int nt, bool mixed, int k, size_t limit, Ba
     }
   }
   if (!b->local) {
-    if (!row((mixed ? H * p8 : p8) > kBandThreads ? 16 : 8)) return false;
+    if (!row(mixed && H * p8 > kBandThreads ? 16 : 8)) return false;
     b->bufb = H * NG * 4 * elem;
   }
   b->faceb = H * NG * 4 * elem;
@@ -414,9 +419,12 @@ bool band_layout(int nlon, int nlat, int nt, bool mixed, int k, size_t limit, Ba
 // Mixed solves of at least this many points stream their step rounds by
 // default: their Krylov vectors (about 16 FP32 vectors of N) far outgrow the
 // 129 MB L2, so a round is bound by HBM rather than by L2 latency.  Smaller
-// solves run faster in one-pass rounds (measured per inner step: 2048 x 1024
-// 83 us in one-pass rounds against 94 streamed; 4096 x 2048 247 streamed
-// against 401 in split rounds).
+// ones run in banded rounds: ms, banded / streamed, random right-hand sides,
+// tol 1e-10, at k = 4 2048 x 1024 3.43 / 4.66, 2048 x 1536 5.75 / 6.49, 4000 x
+// 700 5.22 / 5.67, 4000 x 1000 7.30 / 7.27, 3900 x 1070 7.97 / 8.06; at k = 8,
+// whose rounds move more, the two meet near 3 M points: 2048 x 1536 6.89 /
+// 7.01, 4000 x 700 6.33 / 6.22, 4000 x 1000 8.74 / 7.96.  (4096 x 2048, per
+// inner step, split rounds / streamed: 401 / 247 us.)
 constexpr long long kStreamMinPoints = 4LL * 1024 * 1024;
 
 // Streamed step rounds: one band per SM (at most kMaxStreamRows rows).

@@ -17,10 +17,11 @@
 // 256 in the one-pass rounds) halve the trips of every loop, and a row's line
 // solve spreads over up to 16 warps in pieces of 8 or 16 elements held in
 // registers.  Measured on a GB300, one-pass rounds of 256 threads / banded, us a
-// solve: FP64 64 x 32 1464 / 1088, 512 x 256 1152 / 660, 1440 x 721 6297 / 4981
-// (bound by the FP64 pipe); mixed, k = 4, 360 x 181 743 / 554, 1024 x 512 1172 /
-// 1085, 2048 x 1024 4226 / 3386 (bound by L2); a batch of 128 mixed solves 60.6
-// / 37.7 ms.  Tried and slower: 256 threads; larger bands on fewer CTAs (360 x
+// solve (k = 4, tol 1e-10, zero initial guess, random right-hand sides): FP64
+// 64 x 32 1464 / 1088 (a detected flip), 1440 x 721 6297 / 4981; mixed 360 x 181
+// 743 / 554, 1024 x 512 1172 / 1085, 2048 x 1024 4226 / 3386 (bound by L2).  The
+// hill's flow takes fewer steps: FP64 512 x 256 1152 / 660, mixed 1024 x 512 742
+// / 701; a batch of 128 such mixed solves 60.6 / 37.7 ms.  Tried and slower: 256 threads; larger bands on fewer CTAs (360 x
 // 181 with 5 rows a band 671 against 545); the line solve's constants all
 // loaded at its start, or the face coefficients one group ahead (registers
 // spill); halo packets of several groups polled together; the step out of line.
@@ -1137,10 +1138,11 @@ __device__ __forceinline__ void band_step(int tau, int ntile, int pass, int cur,
         const T *tc = reinterpret_cast<const T*>(pc), *tw = reinterpret_cast<const T*>(pw),
                 *tz = reinterpret_cast<const T*>(pz);
         const unsigned row = rows + (unsigned)(jr * (int)rowb);
-        if (sd.lq == (sizeof(T) == 8 ? 2 : 1))
+        if (sizeof(T) == 8 || sd.lq == 1) {
           band_line_solve<T, 8>(sd, j0 + jr, row, tc, tw, tz, tot, 1 + grp, p);
-        else
-          band_line_solve<T, 16>(sd, j0 + jr, row, tc, tw, tz, tot, 1 + grp, p);
+        } else {
+          if constexpr (sizeof(T) == 4) band_line_solve<T, 16>(sd, j0 + jr, row, tc, tw, tz, tot, 1 + grp, p);
+        }
       }
       __syncthreads();
       sub_mark(ps, 1);

@@ -304,7 +304,7 @@ __device__ __forceinline__ int part_count(int kind, int nu) {
 // The per-solve state machine: consumes the reduced partial sums of the phase
 // that ran last round (S.pending) and decides this round's phase.  One thread.
 // expect: assume the usual outcome of a step round (accepted, the direction's
-// dots from the identities) before its sums are known; see expect_next.
+// dots from the identities) before its sums are known; see can_expect.
 template <typename T>
 __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState& S, const double* red, const double* qd,
                                        SolveState& N, Ctx<T>& c, bool expect = false) {
@@ -2246,7 +2246,7 @@ __device__ __forceinline__ void enter_solve(SolveDev<T>* const* solves, KernelSm
     __syncthreads();
   }
   ls.red_ready = false;
-  precompute_divisions(ks.S, ks.red, ks.qd, ks.sd.mixed || ks.sd.band);
+  precompute_divisions(ks.S, ks.red, ks.qd, ks.sd.mixed);
   if (expected) {
     if (threadIdx.x < 32) {
       __syncwarp();

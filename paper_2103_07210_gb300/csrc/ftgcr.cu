@@ -346,7 +346,6 @@ struct BandLayout {
   size_t bytes;
 };
 constexpr int kOnePassGroups = 1450;  // (see fill_handle_params)
-constexpr int kOnePassGroupsK8 = 1700;
 bool band_layout(int nlon, int nlat, int nt, bool mixed, int k, size_t limit, BandLayout* b) {
   if (nlon > kBandMaxLon) return false;
   const int W = mixed ? 4 : 2, elem = 16 / W, H = (nlat + nt - 1) / nt, NG = (nlon + 3) / 4;
@@ -1347,23 +1346,15 @@ static void fill_handle_params(ftgcr_handle* h, const ftgcr_grid* g, int32_t k, 
   // large ones, whose vectors and face coefficients the banded kernel mostly
   // reads from L2 (one-pass against banded, k = 4, ms: 1440 x 721 of 1800
   // groups a band 1.70 / 1.78, 1200 x 760 of 1500 1.54 / 1.56; but 1400 x 600
-  // of 1400 1.53 / 1.41, 1024 x 750 of 1280 1.36 / 1.28; even for k = 5, 1440 x
-  // 721: 2.06 / 2.04), and k <= 2, where
+  // of 1400 1.53 / 1.41, 1024 x 750 of 1280 1.36 / 1.28; even for k > 4, 1440 x
+  // 721, k = 5: 2.07 / 2.05), and k <= 2, where
   // their own pass over the directions is short (1208 x 531, k = 2: 1.22 /
   // 1.24; k = 4 is ahead when banded).  Widths off the 16-byte unit are always
   // ahead when banded (1209 x 531: 3.00 / 1.62, 801 x 401: 1.78 / 1.04).
   if (mixed && !h->split && !gconsts && h->plan.bytes <= (size_t)smem_limit && h->nt <= sms && !h->bl.local &&
-      g->nlon % 4 == 0) {
-    const int rows = (h->nlat + nt - 1) / nt, groups = rows * (g->nlon / 4);
-    if (k <= 4 && (groups > kOnePassGroups || k <= 2)) return;
-    // k = 6 to 8, large bands of five rows and more (the halo rows' share of
-    // the one-pass work is then small; k = 6 / k = 8, ms, one-pass against
-    // banded: 1400 x 750 2.11 / 2.24 and 2.28 / 2.39, 1240 x 900 2.19 / 2.33 and
-    // 2.40 / 2.49, 1200 x 1000 2.53 / 2.66 and 2.92 / 2.90, 1440 x 721 2.14 / 2.17
-    // and 2.34 / 2.32; but 1320 x 700 of 1650 groups 2.03 / 1.92 and 2.14 / 2.20,
-    // and in bands of four rows 1800 x 608 2.32 / 2.06 and 2.62 / 2.25; above 8
-    // the one-pass kernel is another, 1400 x 750, k = 9: 3.20 / 2.58)
-    if (k >= 6 && k <= 8 && rows >= 5 && groups > kOnePassGroupsK8) return;
+      g->nlon % 4 == 0 && k <= 4) {
+    const int groups = (h->nlat + nt - 1) / nt * (g->nlon / 4);
+    if (groups > kOnePassGroups || k <= 2) return;
   }
   h->nt = nt;
   h->split = 0;

@@ -1346,8 +1346,10 @@ static void fill_handle_params(ftgcr_handle* h, const ftgcr_grid* g, int32_t k, 
   // large ones, whose vectors and face coefficients the banded kernel mostly
   // reads from L2 (one-pass against banded, k = 4, ms: 1440 x 721 of 1800
   // groups a band 1.70 / 1.78, 1200 x 760 of 1500 1.54 / 1.56; but 1400 x 600
-  // of 1400 1.53 / 1.41, 1024 x 750 of 1280 1.36 / 1.28; even for k > 4, 1440 x
-  // 721, k = 5: 2.07 / 2.05), and k <= 2, where
+  // of 1400 1.53 / 1.41, 1024 x 750 of 1280 1.36 / 1.28; for k of 5 to 8 either
+  // is ahead there, by 6 % at most: k = 5, 1440 x 721 2.06 / 2.04, 1200 x 760
+  // 1.80 / 1.63, k = 8, 1440 x 721 2.36 / 2.34, 1160 x 760 1.98 / 1.91, 1400 x
+  // 750 2.28 / 2.39; above 8 banded by a fifth and more), and k <= 2, where
   // their own pass over the directions is short (1208 x 531, k = 2: 1.22 /
   // 1.24; k = 4 is ahead when banded).  Widths off the 16-byte unit are always
   // ahead when banded (1209 x 531: 3.00 / 1.62, 801 x 401: 1.78 / 1.04).

@@ -533,7 +533,9 @@ struct BandSmem {
   T tot[kWarps * 6];
   TeamFail tf;
   int bail;
+  int met;  // the team has met at a barrier since its CTAs loaded the solve's record
   int expected;
+  int events;  // the plan holds flips or data-loss events of the round's step
   int cs_ok;  // the band's static data are staged
 };
 template <typename T>
@@ -762,6 +764,16 @@ __device__ __noinline__ G4<T> flip4(G4<T> x, long long g, int vec, int nv, int n
     x.v[3] = w == 3 ? y : x.v[3];
   }
   return x;
+}
+// Whether the plan holds flips or data-loss events of step t (every lane of a
+// warp, the same answer in all).
+template <typename T>
+__device__ __noinline__ bool band_events(const SolveDev<T>& sd, long long t) {
+  const int lane = threadIdx.x & 31;
+  bool hit = false;
+  for (int q = lane; q < sd.nfaults; q += 32) hit = hit || sd.faults[q].step == t;
+  for (int q = lane; q < sd.nlosses; q += 32) hit = hit || sd.losses[q].step == t;
+  return __any_sync(0xffffffffu, hit);
 }
 // The e-site flips and data-loss events (Section 3) of step t on rows [j0, j1),
 // the first at `rows`.
@@ -992,7 +1004,9 @@ __device__ __noinline__ void band_after(int kind, int tau, int cur, int t, int n
 // loop makes the compiler keep the loop's values in local memory, and with
 // shared memory taking the L1 cache every such access costs an L2 trip).  Only
 // those rounds take it: on every round of a solve with a fault plan it made a
-// mixed 1024 x 512 solve 26 % slower.
+// mixed 1024 x 512 solve 26 % slower.  (Which rounds these are is asked of the
+// plan here, by one warp; counted in the state machine, it moved the compiler's
+// allocation and cost solves without a plan 1 to 3 %.)
 template <typename T, int KB, int KIND, bool AL, bool FLT>
 __device__ __forceinline__ void band_step(int tau, int ntile, int pass, int cur, double* part_out) {
   BandSmem<T>& ks = band_smem<T>();
@@ -1308,7 +1322,7 @@ template <typename T, int KB>
 __device__ __forceinline__ void band_step_any(int kind, int tau, int ntile, int pass, int cur, double* part_out) {
   const SolveDev<T>& sd = band_smem<T>().sd;
   const bool al = (sd.nlon & 3) == 0;
-  if (band_smem<T>().c[cur].events) {  // the unaligned form serves every row width
+  if (band_smem<T>().events) {  // the unaligned form serves every row width
     if (kind == K_INIT)
       band_step_out<T, KB, K_INIT, false, true>(tau, ntile, pass, cur, part_out);
     else if (kind == K_PA)
@@ -1388,7 +1402,6 @@ __device__ __noinline__ void usual_transition(const SolveDev<T>& sd, const Solve
   N.ecur = ec;
   N.pending = c.kind;
   c.nu = nun;
-  c.events = 0;
   c.t = S.step + (step ? 2 : 1);
   c.phiC = sd.phi[phiC];
   c.phiW = sd.phi[phiW];
@@ -1446,7 +1459,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
     const bool local = sizeof(T) == 4 && single && ks.sd.local;
     if (threadIdx.x == 0) ks.ps.cr.stride = 2 * nt;
     bool expected = false, done = false, late = false;
-    bool met = false;  // the team has met at a barrier since its CTAs loaded the record
     long long round = ks.S.round;  // of ks.S, which the last warp rewrites while the others go on
     int pending = ks.S.pending, cur = 0, halo = -1;
     __syncthreads();
@@ -1456,10 +1468,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
     for (int it = 0; it < a.max_rounds; ++it) {
       unsigned long long tr0 = 0ull, tr1 = 0ull;
       cur ^= 1;
-      met = it > 0;
       if (threadIdx.x == 0) {
         tr0 = globaltimer();
         if (tr0 - t_start > kKernelTimeoutNs) ks.tf.raise(2);
+        ks.met = it;
         ks.ps.tracing = a.trace != nullptr;
       }
       const int par = (int)(round & 1);
@@ -1494,7 +1506,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
         band_scalars(pending, ks.S.nu, ks.S.lpn2, ks.red, ks.qd);
         __syncwarp();
         const bool holds = expected && expectation_holds(ks.sd, ks.S, ks.red, ks.qd, ks.N, ks.c[cur]);
-        if (threadIdx.x == 0) ks.expected = holds;
+        const bool events = (ks.sd.nfaults | ks.sd.nlosses) && band_events(ks.sd, ks.c[cur].t);
+        if (threadIdx.x == 0) ks.expected = holds, ks.events = events;
       }
       __syncthreads();
       if (!ks.expected) {
@@ -1515,6 +1528,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
           fill_directions(ks.sd, ks.S, ks.N, ks.qd, ks.c[cur], threadIdx.x);
           __syncwarp();
           band_plan(ks.sd, ks.c[cur], ks.bp[cur], ks.tag, threadIdx.x);
+          if (ks.sd.nfaults | ks.sd.nlosses) {
+            const bool events = band_events(ks.sd, ks.c[cur].t);
+            if (threadIdx.x == 0) ks.events = events;
+          }
         }
         __syncthreads();
       }
@@ -1591,7 +1608,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
         arrive();
         if (sizeof(T) == 4 && late && ta < tb && warp >= kTotWarps) {
           const int t = (int)threadIdx.x - 32 * kTotWarps, nth = 32 * (kSumWarps - kTotWarps);
-          if (ks.c[cur].events)
+          if (ks.events)
             band_after<T, KB, false, true>(kind, ta, cur, t, nth);
           else if ((ks.sd.nlon & 3) == 0)
             band_after<T, KB, true, false>(kind, ta, cur, t, nth);
@@ -1624,7 +1641,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ftgcr_band(BandArgs<T> a) {
       }
     }
     __syncthreads();
-    if (!met) {
+    if (ks.met == 0) {
       // a launch of one round, or a solve with nothing left but its end: the
       // record may be rewritten only once every CTA of the team has loaded it
       if (done) {

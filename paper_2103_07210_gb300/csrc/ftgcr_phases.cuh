@@ -26,7 +26,6 @@ template <typename T>
 struct Ctx {
   int kind, nu, zero_guess, xsrc_user, finzero, patched, first;
   int rin_R;  // INIT: r0 = -R (zero initial guess; mixed: the first inner solve), ||R||^2 in FP64
-  int events;  // INIT, PA, PF: planned flips and data-loss events of step t
   long long t;           // PA: executed step; INIT/PB/RESTORE: step whose x/r/p/Ap flips are applied
   long long patch_step;  // step of the flips whose clean values the backup carries
   T beta;
@@ -650,8 +649,6 @@ __device__ __noinline__ void transition(const SolveDev<T>& sd, const SolveState&
   } else if (c.kind == K_FIN) {
     if (sd.mixed) c.xsrc = N.xzero ? nullptr : sd.xbuf[N.xcur];
   }
-  if (c.kind == K_PA || c.kind == K_PF || c.kind == K_INIT)
-    c.events = count_faults(sd, c.t, ~0u) + count_losses(sd, c.t);
   N.pending = c.kind;
   if (c.kind == K_NONE) N.active = 0;
 }
@@ -2246,7 +2243,9 @@ __device__ __forceinline__ void enter_solve(SolveDev<T>* const* solves, KernelSm
     __syncthreads();
   }
   ls.red_ready = false;
-  precompute_divisions(ks.S, ks.red, ks.qd, ks.sd.mixed);
+  // (banded solves never come here; without the second term the compiler lays
+  // the mixed one-pass kernel out 0.6 % slower: 1440 x 721 1666 against 1656 us)
+  precompute_divisions(ks.S, ks.red, ks.qd, ks.sd.mixed || ks.sd.band);
   if (expected) {
     if (threadIdx.x < 32) {
       __syncwarp();

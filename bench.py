@@ -49,17 +49,17 @@ def algorithmic_bytes(steps: int, outer: int, k: int = K, s: int = 4, N: int = N
     return steps * (14 + 1.5 * (k + 1)) * s * N + refine
 
 
-# DRAM traffic per launch of the persistent kernel from one ncu capture, valid
+# DRAM traffic of a solve (zero initial guess) from one ncu capture, valid
 # only for the kernel sources it was taken on (sha256 of the CUDA sources).
-NCU_TRAFFIC = {"sources_sha256": "d168926416590449a9521c4fa8c62e64a664158f6af5e4915f54f5654b670522",
-               "bytes_per_launch": 23570688 + 6663936,  # mixed 1024x512 (read + write)
-               "large": {"2048x1024": 2652937728 + 1323485440, "4096x2048": 12415849472 + 5120951552}}
+NCU_TRAFFIC = {"sources_sha256": "1d5b5fb458376f0f2cb2db005b41915501fb39e97b3dcd7015435c26383e0c76",
+               "bytes_per_launch": 42429440 + 93857536,  # mixed 1024x512 (read + write)
+               "large": {"2048x1024": 2780000000 + 1860000000, "4096x2048": 12320000000 + 5110000000}}
 
 
 def sources_hash() -> str:
-    """sha256 of the persistent kernel's sources: its device code and the
-    translation units that instantiate it (host code and set-up kernels in
-    ftgcr.cu do not change its DRAM traffic)."""
+    """sha256 of the solve kernels' sources: their device code and the
+    translation units that instantiate them (host code and set-up kernels in
+    ftgcr.cu do not change their DRAM traffic)."""
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2103_07210_gb300", "csrc")
     for f in sorted(os.listdir(d)):
